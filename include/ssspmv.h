@@ -70,11 +70,18 @@ extern "C" {
                                     the batch exceeded the capacity its workspace was sized for
                                     (nothing was computed) */
 
-/* Storing the partial sums of tiles that hold empty rows ("dirty" tiles):
+/* How a product is computed:
+ *  DEFAULT      the library's choice.  With W, S and block_warps 0 as well, FP64
+ *               products go by blocks of rows: a warp takes 32 rows (fewer,
+ *               with several lanes each, when rows are long), so no tile is
+ *               cut out, no row repaired and row_ptr read once; the longest
+ *               rows are left to a second kernel.  Otherwise SPECULATIVE.
+ *  The other two are the segmented sum over tiles, and differ in how tiles
+ *  that hold empty rows ("dirty" tiles) are stored:
  *  SPECULATIVE  the paper's method: kernel (b) stores every segment at its
  *               speculative row tile_offset[t] + s and kernel (c) moves the
  *               partials of dirty tiles to their rows and zeroes empty rows
- *               (Sec. 3.2, checking prediction).  The default.
+ *               (Sec. 3.2, checking prediction).
  *  EXACT        kernel (b) resolves dirty tiles on chip: it already reads the
  *               tile's row pointers, so it stores each partial at the row that
  *               starts at the segment's head and zeroes the empty rows itself;
@@ -116,7 +123,9 @@ typedef struct ssspmv_opts {
  * CUDA runtime instance in the process cannot be recorded from here).  A
  * timer holds `capacity` slots; every call given the timer in opts->timer
  * records 4 events on its stream into the next free slot (before kernel (a),
- * before (b), before (c), after (c)); calls beyond capacity are not timed.
+ * before (b), before (c), after (c); a product by row blocks records its two
+ * kernels as (b) and (c), and nothing between the first two events); calls
+ * beyond capacity are not timed.
  * Not thread safe: one timer per stream. */
 typedef struct ssspmv_timer ssspmv_timer;
 int ssspmv_timer_create(int32_t capacity, ssspmv_timer **out);
@@ -338,8 +347,9 @@ int ssspmv_csr_f64_noalloc(int32_t m, int32_t n, int32_t nnz,
  *     such a row is its y (ssspmv_seam_merge);
  *   - the shard with t0 = 0 also zeroes the leading empty rows [0, r_first).
  * Shards share nothing on the device; the seam records (32 bytes each) are
- * the only exchange.  Their tiles are the unsplit product's tiles, so each
- * tile's arithmetic is the same as in ssspmv_csr_f64.
+ * the only exchange.  Their tiles are the unsplit product's tiles, so with a
+ * tile shape or a variant given each tile's arithmetic is the same as in
+ * ssspmv_csr_f64 (with none, both go by row blocks).
  *   ssspmv_range_bounds   r_first and r_last of [t0, t1) from the device
  *     row_ptr (a search kernel; allocates 8 bytes stream-ordered and
  *     synchronises `stream`).  0 <= t0 <= t1 <= ntiles (ssspmv_plan_shape).
@@ -400,6 +410,8 @@ int ssspmv_csr_f64_host(int32_t m, int32_t n, int32_t nnz,
  *   sync_idx[nbunches]      synchronizer row of each bunch (= tile_offset[w*S])
  *   y_spec[m]               y after kernel (b), before calibration (entries
  *                           kernel (b) does not write are left as y held them)
+ * The artefacts are the segmented sum's whatever the options; y is what
+ * ssspmv_csr_f64 gives with them (by row blocks where it takes those).
  * Synchronises the stream and returns SSSPMV_EDEVICE if a kernel flagged an
  * error. */
 int ssspmv_csr_f64_debug(int32_t m, int32_t n, int32_t nnz,

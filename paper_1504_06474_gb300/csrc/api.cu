@@ -11,6 +11,7 @@
 #include <new>
 
 #include "launch.cuh"
+#include "rowblock.cuh"
 
 namespace ssspmv {
 
@@ -138,6 +139,18 @@ static int make_layout(int32_t m, int32_t nnz, int32_t val_bytes, const ssspmv_o
     return SSSPMV_OK;
 }
 
+// row blocks (rowblock.cuh) are the choice of a caller who asks for no tile
+// shape, bunch size, block size or variant: the segmented sum over tiles
+// remains for those who do.  Their lists live in the sections the tiles'
+// records take otherwise; a layout too small for them keeps the tiles.
+static bool takes_rows(int32_t val_bytes, int32_t m, int32_t nnz, const ssspmv_opts *o,
+                       const Layout &l)
+{
+    if (val_bytes != 8) return false;
+    if (o && (o->W != 0 || o->S != 0 || o->block_warps != 0 || o->variant != 0)) return false;
+    return row_lists_fit(nnz, row_shape(m, nnz), l);
+}
+
 static bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 }  // namespace ssspmv
@@ -223,11 +236,16 @@ static int cached_workspace(size_t need, void *stream, void **ptr, size_t *bytes
     return SSSPMV_OK;
 }
 
+// header: the state of the workspace's header words, kHeaderUnknown for a
+// caller's buffer
+enum { kHeaderUnknown = 0, kHeaderClear = 1 };
+
 static int run_call(int32_t val_bytes, int32_t m, int32_t n, int32_t nnz,
                     const int32_t *row_ptr, const int32_t *col, const void *val, const void *x,
                     void *y, const ssspmv_opts *opts, void *ws, size_t ws_bytes, void *stream,
                     uint32_t *dbg_desc, void *dbg_yspec, Layout *out_layout,
-                    double alpha = 1.0, double beta = 0.0, int axpby = 0)
+                    double alpha = 1.0, double beta = 0.0, int axpby = 0,
+                    int header = kHeaderUnknown, bool tiles_only = false)
 {
     const Prec *pr = prec_for(val_bytes);
     if (!pr) return SSSPMV_EUNSUPPORTED;
@@ -241,6 +259,7 @@ static int run_call(int32_t val_bytes, int32_t m, int32_t n, int32_t nnz,
     if (!ws) {
         rc = cached_workspace(l.total, stream, &ws, &ws_bytes);
         if (rc) return rc;
+        header = kHeaderClear;  // between calls
     }
     if (ws_bytes < l.total || ((uintptr_t)ws & 255u)) return SSSPMV_EWORKSPACE;
     if (opts && opts->variant == SSSPMV_VARIANT_ROWS) {
@@ -293,7 +312,23 @@ static int run_call(int32_t val_bytes, int32_t m, int32_t n, int32_t nnz,
         c.beta = beta;
         c.axpby = 1;
     }
+    if (!tiles_only && takes_rows(val_bytes, m, nnz, opts, l)) {
+        c.rows = 1;
+        if (header != kHeaderClear) {
+            cudaError_t e = cudaMemsetAsync(c.ws + l.off_err, 0, kHeaderBytes, c.stream);
+            if (e != cudaSuccess) return record_cuda_error(e);
+        }
+    }
     return pr->run(c);
+}
+
+// ssspmv_csr_f64 for a workspace whose header words the caller has cleared
+int csr_f64_clear_header(int32_t m, int32_t n, int32_t nnz, const int32_t *row_ptr,
+                         const int32_t *col_idx, const double *val, const double *x, double *y,
+                         const ssspmv_opts *opts, void *ws, size_t ws_bytes, void *stream)
+{
+    return run_call(8, m, n, nnz, row_ptr, col_idx, val, x, y, opts, ws, ws_bytes, stream,
+                    nullptr, nullptr, nullptr, 1.0, 0.0, 0, kHeaderClear);
 }
 
 // ---------------------------------------------------------------------------
@@ -526,6 +561,7 @@ struct ssspmv_plan {
     size_t ws_bytes = 0;
     bool owns_ws = false;
     int exact = 0, block_warps = 0, dev = 0;
+    int rows = 0;  // by row blocks: no partition to keep
 };
 
 int ssspmv_plan_create(int32_t m, int32_t n, int32_t nnz, const int32_t *row_ptr,
@@ -555,6 +591,7 @@ int ssspmv_plan_create(int32_t m, int32_t n, int32_t nnz, const int32_t *row_ptr
     p->lay = l;
     p->exact = (opts && opts->variant == SSSPMV_VARIANT_EXACT) ? 1 : 0;
     p->block_warps = opts ? opts->block_warps : 0;
+    p->rows = takes_rows(val_bytes, m, nnz, opts, l) ? 1 : 0;
     if (workspace && (ws_bytes < l.total || ((uintptr_t)workspace & 255u))) {
         delete p;
         return SSSPMV_EWORKSPACE;
@@ -585,10 +622,11 @@ int ssspmv_plan_create(int32_t m, int32_t n, int32_t nnz, const int32_t *row_ptr
             ssspmv_plan_destroy(p);
             return record_cuda_error(e);
         }
-        launch_partition(row_ptr, m, nnz, l.L, l.ntiles,
-                         reinterpret_cast<int32_t *>(w + l.off_tile_offset),
-                         reinterpret_cast<uint32_t *>(w + l.off_err),
-                         static_cast<cudaStream_t>(stream), partition_method(m, l.ntiles));
+        if (!p->rows)
+            launch_partition(row_ptr, m, nnz, l.L, l.ntiles,
+                             reinterpret_cast<int32_t *>(w + l.off_tile_offset),
+                             reinterpret_cast<uint32_t *>(w + l.off_err),
+                             static_cast<cudaStream_t>(stream), partition_method(m, l.ntiles));
         e = cudaGetLastError();
         if (e != cudaSuccess) {
             ssspmv_plan_destroy(p);
@@ -628,6 +666,7 @@ int ssspmv_plan_execute(ssspmv_plan *p, const int32_t *col_idx, const void *val,
     c.exact = p->exact;
     c.block_warps = p->block_warps;
     c.skip_partition = 1;
+    c.rows = p->rows;
     return pr->run(c);
 }
 
@@ -716,6 +755,7 @@ int ssspmv_plan_execute_axpby(ssspmv_plan *p, const int32_t *col_idx, const void
     c.exact = 1;  // see run_call
     c.block_warps = p->block_warps;
     c.skip_partition = 1;
+    c.rows = p->rows;
     c.alpha = alpha;
     c.beta = beta;
     c.axpby = 1;
@@ -731,7 +771,7 @@ int ssspmv_csr_f64_debug(int32_t m, int32_t n, int32_t nnz, const int32_t *row_p
     if (!workspace) return SSSPMV_EWORKSPACE;  // the artefacts are read back from it
     Layout l;
     int rc = run_call(8, m, n, nnz, row_ptr, col_idx, val, x, y, opts, workspace, ws_bytes, stream,
-                      desc, y_spec, &l);
+                      desc, y_spec, &l, 1.0, 0.0, 0, kHeaderUnknown, true);
     if (rc) return rc;
     if (m == 0) return SSSPMV_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -748,6 +788,14 @@ int ssspmv_csr_f64_debug(int32_t m, int32_t n, int32_t nnz, const int32_t *row_p
                             cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return record_cuda_error(e);
     uint32_t bits = 0;
+    rc = ssspmv_device_status(workspace, ws_bytes, stream, 0, &bits);
+    if (rc) return rc;
+    if (bits) return SSSPMV_EDEVICE;
+    if (!takes_rows(8, m, nnz, opts, l)) return SSSPMV_OK;
+    // ssspmv_csr_f64 with these options goes by row blocks: y is its y
+    rc = run_call(8, m, n, nnz, row_ptr, col_idx, val, x, y, opts, workspace, ws_bytes, stream,
+                  nullptr, nullptr, nullptr);
+    if (rc) return rc;
     rc = ssspmv_device_status(workspace, ws_bytes, stream, 0, &bits);
     if (rc) return rc;
     return bits ? SSSPMV_EDEVICE : SSSPMV_OK;

@@ -20,6 +20,7 @@ struct Call {
     cudaEvent_t *ev = nullptr;       // 4 library-owned events or null
     int exact = 0;                   // dirty tiles store in their true rows
     int block_warps = 0;             // warps per block of kernel (b); 0: the most that fit
+    int rows = 0;                    // by row blocks instead of tiles (rowblock.cuh)
     int skip_partition = 0;          // plan execution: tile offsets already in the workspace
     double alpha = 1.0, beta = 0.0;  // y = alpha A x + beta y when axpby (exact stores)
     int axpby = 0;
@@ -36,9 +37,9 @@ constexpr int kZeroBlocks = 32;
 // finishes (programmatic dependent launch): the kernel calls grid_dep_wait()
 // before it reads anything that kernel wrote.  Kernels (b) and (c) are
 // launched this way, which hides most of a launch's latency.
-template <class... Params, class Arg>
+template <class... Params, class... Args>
 cudaError_t launch_dependent(void (*kernel)(Params...), unsigned grid, unsigned block,
-                             size_t smem, cudaStream_t stream, const Arg &arg)
+                             size_t smem, cudaStream_t stream, const Args &...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -50,7 +51,7 @@ cudaError_t launch_dependent(void (*kernel)(Params...), unsigned grid, unsigned 
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, arg);
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // resident warps per SM of kernel (b) for this tile shape when launched with

@@ -25,17 +25,21 @@ inline int32_t auto_bunch_tiles(int64_t ntiles)
     return (int32_t)(s < 1 ? 1 : (s > kDefaultS ? kDefaultS : s));
 }
 
-// The four words at the front of a workspace (uint32 each):
+// The words at the front of a workspace (uint32 each):
 //   [0] device error bits          cleared by kernel (a)
 //   [1] bunch ticket of kernel (b) cleared by kernel (a)
 //   [2] dirty-tile count           cleared by kernel (a); kernel (b) appends
 //                                  the dirty tiles it leaves to kernel (c)
 //   [3] kernel (b)'s schedule flag set by kernel (a) when it sees runs of
 //                                  empty rows, cleared by kernel (c)
+//   [4,5] lengths of the lists of rows rowblock_kernel leaves to
+//         rowtail_kernel, [6] rowtail_kernel's ticket, [7] its finished
+//         blocks: zero between calls (rowtail_kernel clears them)
 // (a plan execution, which skips kernel (a), clears words 0..2 and keeps the
 // plan's flag)
 constexpr int kWordErr = 0, kWordTicket = 1, kWordDirty = 2, kWordSpread = 3;
-constexpr size_t kHeaderBytes = 16;
+constexpr int kWordLists = 4, kWordTailTicket = 6, kWordTailDone = 7;
+constexpr size_t kHeaderBytes = 32;
 
 struct Layout {
     int32_t W = 0, L = 0, S = 0;

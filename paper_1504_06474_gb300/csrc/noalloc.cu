@@ -40,6 +40,10 @@ namespace ssspmv {
 int record_cuda_error(cudaError_t e);  // api.cu
 int check_csr_args(int32_t m, int32_t n, int32_t nnz, const void *row_ptr, const void *col,
                    const void *val, const void *x, const void *y);  // api.cu
+int csr_f64_clear_header(int32_t m, int32_t n, int32_t nnz, const int32_t *row_ptr,
+                         const int32_t *col_idx, const double *val, const double *x, double *y,
+                         const ssspmv_opts *opts, void *ws, size_t ws_bytes,
+                         void *stream);  // api.cu
 }
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[SSSPMV_NOALLOC_SCRATCH_BYTES];
@@ -96,6 +100,6 @@ extern "C" int ssspmv_csr_f64_noalloc(int32_t m, int32_t n, int32_t nnz, const i
         e = cudaMemsetAsync(scratch, 0, ssspmv::kHeaderBytes, st);
         if (e != cudaSuccess) return ssspmv::record_cuda_error(e);
     }
-    return ssspmv_csr_f64(m, n, nnz, row_ptr, col_idx, val, x, y, opts, scratch,
-                          (size_t)SSSPMV_NOALLOC_SCRATCH_BYTES, stream);
+    return ssspmv::csr_f64_clear_header(m, n, nnz, row_ptr, col_idx, val, x, y, opts, scratch,
+                                        (size_t)SSSPMV_NOALLOC_SCRATCH_BYTES, stream);
 }

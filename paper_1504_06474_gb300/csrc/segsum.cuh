@@ -36,6 +36,10 @@ struct F64 {
     // R-MAT scale 22 kernel (b) 362 -> 350 us; the FP32 forms lose 2-3%)
     static constexpr bool kEarlyLongScan = true;
     static constexpr int kShortRowWarps = 14;  // short rows: keep L1 for the gathers (measured)
+    static constexpr int kRowWarps = 20;  // row blocks: warps per block (96 registers)
+    // row blocks: a group of T entries whose longest lane takes n steps keeps
+    // a lane per row (or G lanes) rather than an even split of its entries
+    __device__ static __forceinline__ bool rows_even(int n, int T) { return n <= (T >> 5) + (T >> 6) + 8; }
     using val_t = double;
     using x_t = double;
     using y_t = double;
@@ -97,6 +101,11 @@ struct CompF32Traits {
     static constexpr int kBatchMaxWarps = 20;  // the batched kernel needs more registers
     static constexpr bool kEarlyLongScan = false;  // see F64
     static constexpr int kShortRowWarps = 16;  // short rows: keep L1 for the gathers (measured)
+    static constexpr int kRowWarps = 24;  // 80 registers
+    __device__ static __forceinline__ bool rows_even(int n, int T)  // see F64
+    {
+        return 16 * n <= (T >> 5) * 28 + 240;
+    }
     using val_t = V;
     using x_t = float;
     using y_t = float;

@@ -1,5 +1,6 @@
 // spmv_f64.cu -- FP64 instantiations (val, x, y and accumulation in double).
 #include "launch.cuh"
+#include "rowblock.cuh"
 
 namespace ssspmv {
 
@@ -24,6 +25,7 @@ int f64_resolve(Layout &l, int32_t S_opt)
 
 int f64_run(Call &c)
 {
+    if (c.rows) return run_rowblock<F64>(c);
     switch (c.lay.W) {
 #define X(w) case w: return run_shape<F64, w>(c);
         SSSPMV_SHAPES(X)

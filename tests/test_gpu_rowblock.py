@@ -1,0 +1,110 @@
+"""The automatic choice (no options: products by blocks of rows) at the sizes
+where it can go wrong: group and copy edges, ragged ends of the arrays, every
+number of lanes per row, groups too uneven for a lane per row, groups too
+large to stage, rows cut into pieces, empty rows everywhere.  Small integers,
+so every sum is exact in any order and y must equal the oracle's row loop;
+one structure of each kind also with real values against 1e-13 * sum|a x|."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1504_06474_gb300 import _build
+    _build.build()
+    return torch.device("cuda:0")
+
+
+def _lens(kind, m, rng):
+    if kind.startswith("const"):
+        return np.full(m, int(kind[5:]))
+    if kind.startswith("upto"):
+        return rng.integers(0, int(kind[4:]) + 1, size=m)
+    if kind == "empty":
+        return np.zeros(m, np.int64)
+    lens = rng.integers(0, 9, size=m) * (rng.random(m) < 0.5)
+    if kind == "uneven":      # a few rows of hundreds among short ones
+        lens[rng.random(m) < 0.05] = 300
+    elif kind == "oversized":  # groups past the staging buffer, rows short of a piece
+        lens[rng.random(m) < 0.03] = 1500
+        lens[m // 2: m // 2 + 20] = 1100
+    elif kind == "pieces":    # rows of one to many pieces, at their edges
+        at = rng.choice(m, size=min(m, 8), replace=False)
+        lens[at] = np.array([2047, 2048, 2049, 4096, 4097, 12000, 20000, 70001])[: at.size]
+    else:                     # "power": row lengths falling by powers
+        lens = np.minimum((2.0 / (rng.random(m) + 1e-4)).astype(np.int64), 9000)
+        lens[rng.random(m) < 0.4] = 0
+    return lens
+
+
+KINDS = ["const1", "const8", "const16", "const27", "const28", "const31", "const60", "const64",
+         "const120", "const250", "const500", "const1100", "upto4", "upto12", "upto40", "upto200",
+         "empty", "uneven", "oversized", "pieces", "power"]
+
+
+def _matrix(kind, m, n, seed, integers=True):
+    rng = np.random.default_rng(seed)
+    rp = np.zeros(m + 1, np.int64)
+    np.cumsum(_lens(kind, m, rng), out=rp[1:])
+    nnz = int(rp[-1])
+    col = rng.integers(0, n, size=nnz).astype(np.int32)
+    if integers:
+        val = rng.integers(-6, 7, size=nnz).astype(float)
+        x = rng.integers(-6, 7, size=n).astype(float)
+    else:
+        val, x = rng.uniform(-1, 1, nnz), rng.uniform(-1, 1, n)
+    return rp.astype(np.int32), col, val, x
+
+
+def _device(dev, arrays):
+    return [torch.as_tensor(a, device=dev) for a in arrays]
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_f64_equals_the_row_loop(dev, kind):
+    from paper_1504_06474_gb300 import ssspmv as C
+    for m in (1, 31, 33, 1000, 9001) + ((800_003,) if kind in ("upto4", "empty", "power") else ()):
+        if kind == "const1100" and m > 1000:
+            continue
+        rp, col, val, x = _matrix(kind, m, 517, seed=m)
+        nnz, want = int(rp[-1]), oracle.spmv(rp, col, val, x)
+        rpd, cd, vd, xd = _device(dev, (rp, col, val, x))
+        # the library's workspace, a caller's (full of ones), and a plan, twice each
+        ws = torch.full((C.ssspmv_workspace_bytes(m, nnz, 8, None),), 255, dtype=torch.uint8,
+                        device=dev)
+        plan = C.ssspmv_plan_create(m, 517, nnz, rpd, 8)
+        try:
+            for call in range(6):
+                y = torch.full((m,), float("nan"), dtype=torch.float64, device=dev)
+                if call < 4:
+                    rc = C.ssspmv_csr_f64(m, 517, nnz, rpd, cd, vd, xd, y,
+                                          workspace=None if call < 2 else ws)
+                else:
+                    rc = C.ssspmv_plan_execute(plan, cd, vd, xd, y)
+                C.check(rc, "call %d" % call)
+                assert np.array_equal(y.cpu().numpy(), want), (kind, m, call)
+            assert C.ssspmv_device_status(ws) == 0
+            # y = 2 A x - 3 y
+            C.check(C.ssspmv_plan_execute_axpby(plan, cd, vd, xd, y, 2.0, -3.0), "axpby")
+            assert np.array_equal(y.cpu().numpy(), -want), (kind, m)
+        finally:
+            C.ssspmv_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("kind", ["upto40", "const64", "uneven", "oversized", "pieces", "power"])
+def test_f64_rounding(dev, kind):
+    from paper_1504_06474_gb300 import ssspmv as C
+    m, n = 20_011, 4001
+    rp, col, val, x = _matrix(kind, m, n, seed=5, integers=False)
+    rpd, cd, vd, xd = _device(dev, (rp, col, val, x))
+    y = torch.full((m,), float("nan"), dtype=torch.float64, device=dev)
+    C.check(C.ssspmv_csr_f64(m, n, int(rp[-1]), rpd, cd, vd, xd, y), "csr")
+    yref, s = oracle.spmv_dot2(rp, col, val, x)
+    assert np.all(np.abs(y.cpu().numpy() - yref) <= 1e-13 * s)
