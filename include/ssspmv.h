@@ -71,7 +71,7 @@ extern "C" {
                                     (nothing was computed) */
 
 /* How a product is computed:
- *  DEFAULT      the library's choice.  With W, S and block_warps 0 as well, FP64
+ *  DEFAULT      the library's choice.  With W, S and block_warps 0 as well,
  *               products go by blocks of rows: a warp takes 32 rows (fewer,
  *               with several lanes each, when rows are long), so no tile is
  *               cut out, no row repaired and row_ptr read once; the longest
@@ -230,11 +230,12 @@ int ssspmv_plan_execute_axpby(ssspmv_plan *plan, const int32_t *col_idx, const v
 void ssspmv_plan_destroy(ssspmv_plan *plan);
 
 /* Batched FP32 products y_i = A_i x_i for `count` matrices of any sizes in
- * one pass: a set-up kernel, kernel (a) over every matrix, ONE persistent
- * launch of kernel (b) over every bunch of every matrix (bunches never cross
- * matrices) and kernel (c) over all of them -- four launches whatever the
- * count, no host synchronisation and no allocation, so the call can be
- * captured in a CUDA graph.  The paper runs one matrix at a time; batching is
+ * one pass: a set-up kernel and the two kernels of the row blocks over every
+ * matrix; with a tile shape or a variant given, a set-up kernel, kernel (a)
+ * over every matrix, ONE persistent launch of kernel (b) over every bunch of
+ * every matrix (bunches never cross matrices) and kernel (c) over all of them.
+ * Three or four launches whatever the count, no host synchronisation and no
+ * allocation, so the call can be captured in a CUDA graph.  The paper runs one matrix at a time; batching is
  * this library's addition.
  *   mats       DEVICE array of `count` descriptors, 8-byte aligned; each
  *              describes one matrix exactly as the single FP32 call takes it
@@ -246,7 +247,7 @@ void ssspmv_plan_destroy(ssspmv_plan *plan);
  *              total_nnz and opts).  A batch that turns out larger computes
  *              nothing and sets SSSPMV_DEV_BATCH.
  *   opts       as for the single calls (one tile shape W and bunch size S for
- *              the whole batch; opts->timer records the four launches as
+ *              the whole batch; opts->timer records the launches as
  *              set-up+(a), (b), (c)).
  * Results equal the single FP32 call's bit for bit for every matrix. */
 typedef struct ssspmv_csr_desc {

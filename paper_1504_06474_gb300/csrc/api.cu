@@ -107,6 +107,12 @@ static int resolve_w(int32_t m, int32_t nnz, int32_t val_bytes, const ssspmv_opt
     return SSSPMV_OK;
 }
 
+// whether the caller leaves the way to compute to the library
+static bool automatic(const ssspmv_opts *o)
+{
+    return !o || (o->W == 0 && o->S == 0 && o->block_warps == 0 && o->variant == 0);
+}
+
 // device-independent part of the layout: tile shape, tile count, bunch cap
 static int make_layout(int32_t m, int32_t nnz, int32_t val_bytes, const ssspmv_opts *o, Layout &l)
 {
@@ -136,6 +142,12 @@ static int make_layout(int32_t m, int32_t nnz, int32_t val_bytes, const ssspmv_o
     const int32_t S = (o && o->S > 0) ? o->S : auto_bunch_tiles(l.ntiles);
     l.nbunch_cap = (l.ntiles + S - 1) / S;
     carve(l);
+    // the lists of the row blocks outgrow the records of BF16's longer tiles
+    if (val_bytes == 2 && automatic(o)) {
+        const RowShape s = row_shape(m, nnz);
+        const size_t need = l.off_tile_offset + row_lists(nnz, s.cap, s.piece).bytes;
+        if (l.total < need) l.total = align256(need);
+    }
     return SSSPMV_OK;
 }
 
@@ -143,12 +155,9 @@ static int make_layout(int32_t m, int32_t nnz, int32_t val_bytes, const ssspmv_o
 // shape, bunch size, block size or variant: the segmented sum over tiles
 // remains for those who do.  Their lists live in the sections the tiles'
 // records take otherwise; a layout too small for them keeps the tiles.
-static bool takes_rows(int32_t val_bytes, int32_t m, int32_t nnz, const ssspmv_opts *o,
-                       const Layout &l)
+static bool takes_rows(int32_t m, int32_t nnz, const ssspmv_opts *o, const Layout &l)
 {
-    if (val_bytes != 8) return false;
-    if (o && (o->W != 0 || o->S != 0 || o->block_warps != 0 || o->variant != 0)) return false;
-    return row_lists_fit(nnz, row_shape(m, nnz), l);
+    return automatic(o) && row_lists_fit(nnz, row_shape(m, nnz), l);
 }
 
 static bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
@@ -312,7 +321,7 @@ static int run_call(int32_t val_bytes, int32_t m, int32_t n, int32_t nnz,
         c.beta = beta;
         c.axpby = 1;
     }
-    if (!tiles_only && takes_rows(val_bytes, m, nnz, opts, l)) {
+    if (!tiles_only && takes_rows(m, nnz, opts, l)) {
         c.rows = 1;
         if (header != kHeaderClear) {
             cudaError_t e = cudaMemsetAsync(c.ws + l.off_err, 0, kHeaderBytes, c.stream);
@@ -518,6 +527,7 @@ static int make_batch_layout(int32_t count, int64_t total_nnz, int32_t val_bytes
     // global tile and bunch numbers are 32-bit in the kernels
     if (total_nnz / (32 * W) + count > (int64_t)SSSPMV_MAX_DIM) return SSSPMV_EINVAL;
     batch_layout(count, total_nnz, W, S, l);
+    if (automatic(o)) batch_rows_layout(count, kMinCap, kMinPiece, l);
     return SSSPMV_OK;
 }
 
@@ -591,7 +601,7 @@ int ssspmv_plan_create(int32_t m, int32_t n, int32_t nnz, const int32_t *row_ptr
     p->lay = l;
     p->exact = (opts && opts->variant == SSSPMV_VARIANT_EXACT) ? 1 : 0;
     p->block_warps = opts ? opts->block_warps : 0;
-    p->rows = takes_rows(val_bytes, m, nnz, opts, l) ? 1 : 0;
+    p->rows = takes_rows(m, nnz, opts, l) ? 1 : 0;
     if (workspace && (ws_bytes < l.total || ((uintptr_t)workspace & 255u))) {
         delete p;
         return SSSPMV_EWORKSPACE;
@@ -791,7 +801,7 @@ int ssspmv_csr_f64_debug(int32_t m, int32_t n, int32_t nnz, const int32_t *row_p
     rc = ssspmv_device_status(workspace, ws_bytes, stream, 0, &bits);
     if (rc) return rc;
     if (bits) return SSSPMV_EDEVICE;
-    if (!takes_rows(8, m, nnz, opts, l)) return SSSPMV_OK;
+    if (!takes_rows(m, nnz, opts, l)) return SSSPMV_OK;
     // ssspmv_csr_f64 with these options goes by row blocks: y is its y
     rc = run_call(8, m, n, nnz, row_ptr, col_idx, val, x, y, opts, workspace, ws_bytes, stream,
                   nullptr, nullptr, nullptr);

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include "launch.cuh"
+#include "rowblock.cuh"
 
 namespace ssspmv {
 
@@ -58,6 +59,17 @@ __device__ __forceinline__ int64_t block_exclusive_scan(int64_t v, int64_t *warp
     return before;
 }
 
+__device__ __forceinline__ bool valid_desc(const DescView &d)
+{
+    if (d.reserved != 0 || d.m < 0 || d.n < 0 || d.nnz < 0) return false;
+    if (d.m > SSSPMV_MAX_DIM || d.nnz > SSSPMV_MAX_DIM) return false;
+    if (d.m == 0) return d.nnz == 0;
+    if (!d.row_ptr || !d.y) return false;
+    if (d.nnz > 0 && (!d.col || !d.val || !d.x || d.n == 0)) return false;
+    if (d.nnz > 0 && ((((uintptr_t)d.col) | ((uintptr_t)d.val)) & 15u)) return false;
+    return true;
+}
+
 // One block.  Checks every descriptor (an invalid one is skipped as an empty
 // matrix and flagged), numbers the tiles, bunches and rows of the batch, and
 // writes the records and totals {tiles, bunches} (totals 0 when the batch
@@ -80,20 +92,11 @@ __global__ void __launch_bounds__(kPrepThreads)
     const int32_t per = (count + kPrepThreads - 1) / kPrepThreads;
     const int32_t i0 = threadIdx.x * per;
     const int32_t i1 = (i0 + per < count) ? i0 + per : count;
-    auto valid = [&](const DescView &d) {
-        if (d.reserved != 0 || d.m < 0 || d.n < 0 || d.nnz < 0) return false;
-        if (d.m > SSSPMV_MAX_DIM || d.nnz > SSSPMV_MAX_DIM) return false;
-        if (d.m == 0) return d.nnz == 0;
-        if (!d.row_ptr || !d.y) return false;
-        if (d.nnz > 0 && (!d.col || !d.val || !d.x || d.n == 0)) return false;
-        if (d.nnz > 0 && ((((uintptr_t)d.col) | ((uintptr_t)d.val)) & 15u)) return false;
-        return true;
-    };
     int64_t nt = 0, nbn = 0, nr = 0;
     bool bad = false;
     for (int32_t i = i0; i < i1; ++i) {
         const DescView d = desc[i];
-        if (!valid(d)) {
+        if (!valid_desc(d)) {
             bad = true;
             continue;
         }
@@ -110,7 +113,7 @@ __global__ void __launch_bounds__(kPrepThreads)
     const bool fits = tot_t <= cap_tiles && tot_b <= cap_bunches;
     for (int32_t i = i0; i < i1; ++i) {
         DescView d = desc[i];
-        if (!valid(d)) d = DescView{0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, nullptr};
+        if (!valid_desc(d)) d = DescView{0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, nullptr};
         const int64_t t = ((int64_t)d.nnz + L - 1) / L;
         BatchMat r;
         r.val = d.val;
@@ -293,9 +296,108 @@ int run_batched_shape(int32_t count, const void *desc, const BatchLayout &l, uns
     return SSSPMV_OK;
 }
 
+// Set-up of a batch by row blocks (one block): checks the descriptors as above,
+// numbers the batch's units of rows and writes the records.  The capacity is
+// counted in tiles too, so the two ways accept the same batches.
+__global__ void __launch_bounds__(kPrepThreads)
+    batch_rows_prep_kernel(const DescView *__restrict__ desc, int32_t count, int32_t L,
+                           int64_t cap_tiles, RowMat *__restrict__ mats, uint32_t *head)
+{
+    __shared__ int64_t warp_sums[32];
+    if (threadIdx.x < 8) head[threadIdx.x] = 0u;
+    __syncthreads();
+    const int32_t per = (count + kPrepThreads - 1) / kPrepThreads;
+    const int32_t i0 = threadIdx.x * per;
+    const int32_t i1 = (i0 + per < count) ? i0 + per : count;
+    int64_t nt = 0, nu = 0;
+    bool bad = false;
+    for (int32_t i = i0; i < i1; ++i) {
+        const DescView d = desc[i];
+        if (!valid_desc(d)) {
+            bad = true;
+            continue;
+        }
+        nt += ((int64_t)d.nnz + L - 1) / L;
+        nu += row_units(d.m, row_shape(d.m, d.nnz)).nunits;
+    }
+    if (bad) atomicOr(head + kWordErr, SSSPMV_DEV_BATCH);
+    int64_t tot_t = 0, tot_u = 0;
+    block_exclusive_scan(nt, warp_sums, &tot_t);
+    int64_t ub = block_exclusive_scan(nu, warp_sums, &tot_u);
+    // (units are numbered in 32 bits)
+    const bool fits = tot_t <= cap_tiles && tot_u <= (int64_t)SSSPMV_MAX_DIM;
+    for (int32_t i = i0; i < i1; ++i) {
+        DescView d = desc[i];
+        if (!valid_desc(d) || !fits)
+            d = DescView{0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, nullptr};
+        const RowShape s = row_shape(d.m, d.nnz);
+        const RowUnits u = row_units(d.m, s);
+        RowMat r;
+        r.val = d.val;
+        r.col = d.col;
+        r.row_ptr = d.row_ptr;
+        r.x = d.x;
+        r.y = d.y;
+        r.m = d.m;
+        r.nnz = d.nnz;
+        r.unit_base = fits ? (int32_t)ub : 0;
+        r.nbig = u.nbig;
+        r.cap = s.cap;
+        r.packed = s.gs | (s.us << 8) | (s.piece << 16);
+        mats[i] = r;
+        ub += u.nunits;
+    }
+    if (threadIdx.x == 0) {
+        head[kBatchWordUnits] = fits ? (uint32_t)tot_u : 0u;
+        if (!fits) atomicOr(head + kWordErr, SSSPMV_DEV_BATCH);
+    }
+}
+
+// the batch by row blocks: set-up, (r1) over every unit of every matrix, (r2)
+static int run_batched_rows(int32_t count, const void *desc, const BatchLayout &l,
+                            unsigned char *ws, cudaStream_t stream, cudaEvent_t *ev)
+{
+    using P = F32C;
+    cudaError_t e = cudaSuccess;
+    RowArgs a = {};
+    a.head = reinterpret_cast<uint32_t *>(ws + l.off_err);
+    a.ranges = reinterpret_cast<int2 *>(ws + l.off_ranges);
+    a.pieces = reinterpret_cast<int2 *>(ws + l.off_pieces);
+    a.parts = reinterpret_cast<double *>(ws + l.off_parts);
+    a.arrived = reinterpret_cast<uint32_t *>(ws + l.off_arrived);
+    a.max_ranges = (int32_t)l.cap_ranges;
+    a.max_pieces = (int32_t)l.cap_pieces;
+    a.alpha = 1.0;
+    a.mats = reinterpret_cast<RowMat *>(ws + l.off_rmats);
+    a.count = count;
+    a.total_units = reinterpret_cast<int32_t *>(a.head + kBatchWordUnits);
+    a.range_mat = reinterpret_cast<int32_t *>(ws + l.off_rmat);
+    a.piece_mat = reinterpret_cast<int32_t *>(ws + l.off_pmat);
+    if (ev && (e = cudaEventRecord(ev[0], stream)) != cudaSuccess) return record_cuda_error(e);
+    batch_rows_prep_kernel<<<1, kPrepThreads, 0, stream>>>(
+        static_cast<const DescView *>(desc), count, l.L, l.cap_tiles,
+        reinterpret_cast<RowMat *>(ws + l.off_rmats), a.head);
+    if (ev && (e = cudaEventRecord(ev[1], stream)) != cudaSuccess) return record_cuda_error(e);
+    Call c;
+    c.stream = stream;
+    a.shape.cap = kStageMax;  // any matrix's groups fit
+    a.nnz = 0x7fffffff;       // (the stages' share of shared memory is the usual one)
+    a.nunits = 0x7fffffff;    // known on the device only: all of the GPU
+    int rc = launch_rowblock<P, true, true>(c, a);
+    if (rc) return rc;
+    if (ev && (e = cudaEventRecord(ev[2], stream)) != cudaSuccess) return record_cuda_error(e);
+    rc = launch_rowtail<P, 4, 3, true>(c, a);
+    if (rc) return rc;
+    if (ev && (e = cudaEventRecord(ev[3], stream)) != cudaSuccess) return record_cuda_error(e);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return record_cuda_error(e);
+    return SSSPMV_OK;
+}
+
 int f32_run_batched(int32_t count, const void *desc, const BatchLayout &l, unsigned char *ws,
                     cudaStream_t stream, int exact, int block_warps, cudaEvent_t *ev)
 {
+    if (l.rows) return run_batched_rows(count, desc, l, ws, stream, ev);
     switch (l.W) {
 #define X(w)                                                                                   \
     case w: return run_batched_shape<F32C, w>(count, desc, l, ws, stream, exact, block_warps, ev);

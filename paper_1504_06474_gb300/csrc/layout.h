@@ -75,18 +75,25 @@ inline void carve(Layout &l)
 }
 
 // workspace carve-up of a batch (one 64-byte record per matrix, BatchMat)
-constexpr size_t kBatchMatBytes = 64;
+constexpr size_t kBatchMatBytes = 64, kRowMatBytes = 64;
 
 struct BatchLayout {
     int32_t W = 0, L = 0, S = 0;
     int64_t cap_tiles = 0, cap_bunches = 0;
+    // by row blocks (rowblock.cuh): the records, and the lists of rows left to
+    // the second kernel
+    int32_t rows = 0;
+    int64_t cap_ranges = 0, cap_pieces = 0;
+    size_t off_rmats = 0, off_ranges = 0, off_rmat = 0, off_pieces = 0, off_pmat = 0,
+           off_parts = 0, off_arrived = 0;
     size_t off_err = 0, off_mats = 0, off_toff = 0, off_info = 0, off_dirty = 0, off_bmat = 0,
            off_sidx = 0, off_sval = 0, off_tval = 0, off_tflag = 0, total = 0;
 };
 
 // the words at the front of a batch workspace: error bits, bunch ticket,
-// totals {tiles, bunches} (written by the set-up kernel), dirty-tile count
-constexpr int kBatchWordDirty = 4;
+// totals {tiles, bunches} (written by the set-up kernel), dirty-tile count; by
+// row blocks: error bits, -, units, -, and the list words of a single call
+constexpr int kBatchWordDirty = 4, kBatchWordUnits = 2;
 
 inline void batch_layout(int32_t count, int64_t total_nnz, int32_t W, int32_t S, BatchLayout &l)
 {
@@ -117,6 +124,31 @@ inline void batch_layout(int32_t count, int64_t total_nnz, int32_t W, int32_t S,
     o = align256(o + sizeof(double) * nb);
     l.off_tflag = o;
     o = align256(o + sizeof(int32_t) * nb);
+    l.total = o;
+}
+
+// adds the row blocks' sections: the batch's entries are at most
+// cap_tiles * L, groups of more than 2 * min_cap of them are listed, in pieces
+// of at least 2^min_piece
+inline void batch_rows_layout(int32_t count, int32_t min_cap, int32_t min_piece, BatchLayout &l)
+{
+    const int64_t nnz = l.cap_tiles * l.L;
+    l.rows = 1;
+    l.cap_ranges = nnz / (2 * min_cap) + (nnz >> min_piece) + count + 1;
+    l.cap_pieces = ((2 * nnz) >> min_piece) + count + 1;
+    size_t o = l.total;
+    auto take = [&](size_t bytes) {
+        const size_t at = o;
+        o = align256(o + bytes);
+        return at;
+    };
+    l.off_rmats = take(kRowMatBytes * (size_t)(count > 0 ? count : 1));
+    l.off_ranges = take(8 * (size_t)l.cap_ranges);
+    l.off_rmat = take(4 * (size_t)l.cap_ranges);
+    l.off_pieces = take(8 * (size_t)l.cap_pieces);
+    l.off_pmat = take(4 * (size_t)l.cap_pieces);
+    l.off_parts = take(8 * (size_t)l.cap_pieces);
+    l.off_arrived = take(4 * (size_t)l.cap_pieces);
     l.total = o;
 }
 

@@ -50,7 +50,7 @@ struct RowShape {
 // 17 warps with stages this large leave 60 KB of L1
 constexpr int32_t kStageMax = 888;
 
-constexpr int32_t kMinCap = 640;
+constexpr int32_t kMinCap = 640, kMinPiece = 10;
 
 __host__ __device__ inline RowShape row_shape(int32_t m, int32_t nnz)
 {
@@ -71,7 +71,7 @@ __host__ __device__ inline RowShape row_shape(int32_t m, int32_t nnz)
     if (cap < kMinCap) cap = kMinCap;
     if (cap > kStageMax) cap = kStageMax;
     s.cap = (int32_t)cap;
-    s.piece = nnz <= 15000000 ? 10 : 11;
+    s.piece = nnz <= 15000000 ? kMinPiece : kMinPiece + 1;
     return s;
 }
 
@@ -100,6 +100,37 @@ __host__ __device__ inline RowLists row_lists(int64_t nnz, int32_t cap, int32_t 
     return l;
 }
 
+// one matrix of a batch (filled on the device from the caller's descriptors by
+// the batch set-up kernel)
+struct RowMat {
+    const void *val;
+    const int32_t *col;
+    const int32_t *row_ptr;
+    const void *x;
+    void *y;
+    int32_t m, nnz;
+    int32_t unit_base;  // the batch's number of its first unit
+    int32_t nbig;       // see RowArgs
+    int32_t cap;        // its shape: cap, and gs | us << 8 | piece << 16
+    int32_t packed;
+};
+static_assert(sizeof(RowMat) == kRowMatBytes, "RowMat is one 64-byte record");
+
+// units of rows of a matrix: three quarters of the rows in units of several
+// groups, the rest one group each (they even out the end of the launch)
+struct RowUnits {
+    int32_t nbig, nunits;
+};
+
+__host__ __device__ inline RowUnits row_units(int32_t m, const RowShape &s)
+{
+    const int32_t rows = 32 >> s.gs, big_rows = rows << s.us;
+    RowUnits u;
+    u.nbig = s.us > 0 ? (int32_t)((int64_t)m * 3 / 4 / big_rows) : 0;
+    u.nunits = u.nbig + (int32_t)(((int64_t)m - (int64_t)u.nbig * big_rows + rows - 1) / rows);
+    return u;
+}
+
 struct RowArgs {
     const int32_t *row_ptr;
     const int32_t *col;
@@ -117,6 +148,11 @@ struct RowArgs {
     RowShape shape;
     double alpha, beta;
     int32_t axpby;
+    // batches: the matrices, the batch's units, and the matrix of each list entry
+    const RowMat *mats = nullptr;
+    int32_t count = 0;
+    const int32_t *total_units = nullptr;
+    int32_t *range_mat = nullptr, *piece_mat = nullptr;
 };
 
 // ---------------------------------------------------------------------------
@@ -135,9 +171,9 @@ __device__ __forceinline__ typename P::acc_t lane_dot(const typename P::val_t *v
     using X = typename P::x_t;
     using A = typename P::acc_t;
     const int st = G > 0 ? G : stride;
-    A acc = P::zero();
     // shared index of the lane's i-th entry
     auto at = [&](int i) { return ROT ? (i + rot < n ? i + rot : i + rot - n) * st : i * st; };
+    A acc = P::zero();
     int i = 0;
     for (; i + UN <= nmin; i += UN) {
         X xv[UN];
@@ -182,7 +218,7 @@ __device__ __forceinline__ typename P::acc_t even_split(
 {
     using X = typename P::x_t;
     using A = typename P::acc_t;
-    constexpr int UN = 4;
+    constexpr int UN = P::kSplitBatch;
     const int lane = threadIdx.x & 31;
     const uint32_t hb = sc->heads[lane];
     const int c = __popc(hb);
@@ -196,7 +232,7 @@ __device__ __forceinline__ typename P::acc_t even_split(
     cs += lane * C;
     A sum = P::zero(), pre = P::zero();
     int seg = idx0 - 1;
-    X xa[UN], xb[UN];
+    X xa[UN];
     auto gather = [&](X (&xv)[UN], int i) {
 #pragma unroll
         for (int k = 0; k < UN; ++k)
@@ -215,13 +251,10 @@ __device__ __forceinline__ typename P::acc_t even_split(
             if (i + k < n) sum = P::fma(vs[i + k], xv[k], sum);
         }
     };
-    gather(xa, 0);
 #pragma unroll 1
-    for (int i = 0; i < C; i += 2 * UN) {
-        gather(xb, i + UN);
+    for (int i = 0; i < C; i += UN) {
+        gather(xa, i);
         fmas(xa, i);
-        gather(xa, i + 2 * UN);
-        fmas(xb, i + UN);
     }
     if (c == 0) pre = sum;  // no head: part of an earlier lane's segment
     const bool has = c > 0;
@@ -250,10 +283,10 @@ __device__ __forceinline__ typename P::acc_t even_split(
 
 // a group that is not staged: its rows go to the lists (r2) works on.  Lane l
 // holds row row0 + l of the group, len entries (0 past the group's rows).
-static __device__ __noinline__ void list_group(const RowArgs &a, int32_t row0, int32_t rows, int32_t len)
+static __device__ __noinline__ void list_group(const RowArgs &a, int32_t mat, int32_t pl,
+                                               int32_t row0, int32_t rows, int32_t len)
 {
     const int lane = threadIdx.x & 31;
-    const int32_t pl = a.shape.piece;
     const bool valid = lane < rows;
     const bool isl = valid && len > (1 << pl);
     const int32_t plain = (valid && !isl) ? len : 0;
@@ -278,7 +311,9 @@ static __device__ __noinline__ void list_group(const RowArgs &a, int32_t row0, i
     if (lead) {
         const unsigned above = lane == 31 ? 0u : leads & ~((2u << lane) - 1u);
         const int next = above ? __ffs(above) - 1 : rows;
-        a.ranges[rbase + __popc(leads & ((1u << lane) - 1u))] = make_int2(row0 + lane, next - lane);
+        const int32_t at = rbase + __popc(leads & ((1u << lane) - 1u));
+        a.ranges[at] = make_int2(row0 + lane, next - lane);
+        if (a.range_mat) a.range_mat[at] = mat;
     }
     unsigned todo = __ballot_sync(FULL, isl);
     while (todo) {
@@ -287,19 +322,31 @@ static __device__ __noinline__ void list_group(const RowArgs &a, int32_t row0, i
         const int32_t n = __shfl_sync(FULL, np, src);
         const int32_t at = pbase + __shfl_sync(FULL, pincl, src) - n;
         if (lane == 0) a.arrived[at] = 0u;
-        for (int32_t p = lane; p < n; p += 32) a.pieces[at + p] = make_int2(row0 + src, p);
+        for (int32_t p = lane; p < n; p += 32) {
+            a.pieces[at + p] = make_int2(row0 + src, p);
+            if (a.piece_mat) a.piece_mat[at + p] = mat;
+        }
     }
 }
 
 // ---------------------------------------------------------------------------
 // (r1)
 
+// what is stored in y[row] for a row's sum v (alpha and beta: FP64 only)
+template <class Y>
+__device__ __forceinline__ Y row_value(const RowArgs &a, const Y *y, int32_t row, Y v)
+{
+    if constexpr (sizeof(Y) == sizeof(double))
+        return scaled_store_value(y, row, v, a.alpha, a.beta, a.axpby);
+    else return v;
+}
+
 // copies of the entries [b, e) into a warp's stage (all lanes call it); entry
 // k lands at index k - (b & ~7)
 template <class V>
 __device__ __forceinline__ void stage_copy(unsigned char *st, int32_t col_off, uint64_t *bar,
                                            const V *val, const int32_t *col, int32_t nnz, int32_t b,
-                                           int32_t e)
+                                           int32_t e, uint64_t pol)
 {
     const int lane = threadIdx.x & 31;
     const int32_t b8 = b & ~7;
@@ -307,7 +354,6 @@ __device__ __forceinline__ void stage_copy(unsigned char *st, int32_t col_off, u
     if (e8 > nnz) e8 = nnz & ~7;  // the last entries of the arrays: below
     const int32_t n = e8 > b8 && e > b ? e8 - b8 : 0;
     if (lane == 0) {
-        const uint64_t pol = policy_evict_first();
         fence_proxy_async_smem();
         mbar_arrive_expect_tx(bar, (uint32_t)n * (uint32_t)(sizeof(V) + 4));
         if (n > 0) {
@@ -330,7 +376,7 @@ __device__ __forceinline__ int32_t inside(int32_t p, int32_t b, int32_t e)
     return p < b ? b : (p > e ? e : p);
 }
 
-template <class P, bool MULTI>
+template <class P, bool MULTI, bool BATCHED = false>
 __global__ void __launch_bounds__(P::kRowWarps * 32, 1)
     rowblock_kernel(const RowArgs a, int32_t stage_bytes, int32_t col_off)
 {
@@ -353,18 +399,30 @@ __global__ void __launch_bounds__(P::kRowWarps * 32, 1)
     __syncthreads();
     grid_dep_wait();  // everything read below may come from the kernel before
     grid_dep_trigger();
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.head[kWordErr] = 0u;
+    if (!BATCHED && blockIdx.x == 0 && threadIdx.x == 0) a.head[kWordErr] = 0u;
 
+    // the current unit's matrix (in a batch: loaded again when it changes)
     const X *__restrict__ x = static_cast<const X *>(a.x);
     const V *__restrict__ val = static_cast<const V *>(a.val);
     const int32_t *__restrict__ col = a.col;
     Y *__restrict__ y = static_cast<Y *>(a.y);
-    const int32_t m = a.m, nnz = a.nnz, cap = a.shape.cap;
-    const int gs = MULTI ? a.shape.gs : 0;
-    const int32_t rows = 32 >> gs;  // per group
-    const int sub = lane & ((1 << gs) - 1);
-    const int lrow = lane >> gs;  // the lane's row in its group
-    const uint64_t pol_keep = policy_evict_last();
+    int32_t m = a.m, nnz = a.nnz, cap = a.shape.cap, piece = a.shape.piece;
+    int gs = MULTI ? a.shape.gs : 0;
+    auto load_matrix = [&](int32_t mi) {
+        const RowMat *mm = a.mats + mi;
+        val = static_cast<const V *>(ldg_ptr(&mm->val));
+        x = static_cast<const X *>(ldg_ptr(&mm->x));
+        y = static_cast<Y *>(ldg_ptr(const_cast<void *const *>(&mm->y)));
+        col = ldg_ptr(&mm->col);
+        m = __ldg(&mm->m);
+        nnz = __ldg(&mm->nnz);
+        cap = __ldg(&mm->cap);
+        const int32_t p = __ldg(&mm->packed);
+        gs = p & 255;
+        piece = p >> 16;
+    };
+    const int32_t nunits = BATCHED ? __ldg(a.total_units) : a.nunits;
+    const uint64_t pol_keep = policy_evict_last(), pol_stream = policy_evict_first();
 
     // the block's next unit of rows [r0, r0 + nr): several groups at a time
     // first, single ones towards the end; its row pointers are loaded into
@@ -372,34 +430,51 @@ __global__ void __launch_bounds__(P::kRowWarps * 32, 1)
     constexpr int NP = kUnitRowsMax / 32 + 1;
     struct Unit {
         int32_t r0, nr;
+        int32_t mat;
         int32_t rp[NP];
     };
+    int32_t at_mat = 0;  // the block's tickets only grow, and with them the matrix
     auto next_unit = [&]() -> Unit {
         int32_t t = 0;
         if (lane == 0) t = atomicAdd(&s_ticket, 1);
         t = __shfl_sync(FULL, t, 0);
-        const int64_t u = (int64_t)t * gridDim.x + blockIdx.x;
+        const int64_t u64 = (int64_t)t * gridDim.x + blockIdx.x;
         Unit q;
         q.r0 = -1;
         q.nr = 0;
-        if (u >= a.nunits) return q;
-        const int32_t big = rows << a.shape.us;
-        if (u < a.nbig) {
-            q.r0 = (int32_t)u * big;
+        q.mat = 0;
+        if (u64 >= nunits) return q;
+        int32_t u = (int32_t)u64, um = m, ugs = gs, us = a.shape.us, nbig = a.nbig;
+        const int32_t *row_ptr = a.row_ptr;
+        if constexpr (BATCHED) {
+            while (at_mat + 1 < a.count && u >= __ldg(&a.mats[at_mat + 1].unit_base)) ++at_mat;
+            const RowMat *mm = a.mats + at_mat;
+            row_ptr = ldg_ptr(&mm->row_ptr);
+            um = __ldg(&mm->m);
+            u -= __ldg(&mm->unit_base);
+            nbig = __ldg(&mm->nbig);
+            const int32_t p = __ldg(&mm->packed);
+            ugs = p & 255;
+            us = (p >> 8) & 255;
+            q.mat = at_mat;
+        }
+        const int32_t rows = 32 >> ugs, big = rows << us;
+        if (u < nbig) {
+            q.r0 = u * big;
             q.nr = big;
         } else {
-            q.r0 = a.nbig * big + ((int32_t)u - a.nbig) * rows;
+            q.r0 = nbig * big + (u - nbig) * rows;
             q.nr = rows;
         }
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
             const int32_t r = q.r0 + 32 * i + lane;
-            if (32 * i <= q.nr) q.rp[i] = __ldg(a.row_ptr + (r < m ? r : m));
+            if (32 * i <= q.nr) q.rp[i] = __ldg(row_ptr + (r < um ? r : um));
         }
         return q;
     };
     auto store = [&](int32_t row, A v) {
-        y[row] = scaled_store_value(y, row, P::out(v), a.alpha, a.beta, a.axpby);
+        y[row] = row_value(a, y, row, P::out(v));
     };
 
     // One stage per warp, and as many warps as shared memory holds: a warp
@@ -408,7 +483,12 @@ __global__ void __launch_bounds__(P::kRowWarps * 32, 1)
     uint32_t phase = 0;  // parity of the stage's next completion
     Unit cur = next_unit();
     const int32_t *const rp = sc->rp;
+    int32_t mat = -1;
     while (cur.nr > 0) {
+        if (BATCHED && cur.mat != mat) load_matrix(mat = cur.mat);
+        const int32_t rows = 32 >> gs;  // per group
+        const int sub = lane & ((1 << gs) - 1);
+        const int lrow = lane >> gs;  // the lane's row in its group
 #pragma unroll
         for (int i = 0; i < NP; ++i)
             if (32 * i + lane <= cur.nr) sc->rp[32 * i + lane] = cur.rp[i];
@@ -424,10 +504,11 @@ __global__ void __launch_bounds__(P::kRowWarps * 32, 1)
             const int32_t g0 = inside(rp[j], b, e), ge = inside(rp[j + rows], g0, e);
             const int32_t T = ge - g0;
             if (T > 2 * cap) {
-                const int32_t rs = inside(rp[j + (lane < rows ? lane : 0)], g0, ge);
-                const int32_t re = inside(rp[j + (lane < rows ? lane : 0) + 1], rs, ge);
+                const int32_t l = lane < rows ? lane : 0;
+                const int32_t rs = inside(rp[j + l], g0, ge), re = inside(rp[j + l + 1], rs, ge);
                 const int32_t left = m - (cur.r0 + j);
-                list_group(a, cur.r0 + j, left < rows ? left : rows, lane < rows ? re - rs : 0);
+                list_group(a, cur.mat, piece, cur.r0 + j, left < rows ? left : rows,
+                           lane < rows ? re - rs : 0);
                 j += rows;
                 continue;
             }
@@ -449,7 +530,7 @@ __global__ void __launch_bounds__(P::kRowWarps * 32, 1)
                 }
             }
             __syncwarp();  // every lane is done with the copy before
-            stage_copy(st, col_off, &sc->bar, val, col, nnz, ts, te);
+            stage_copy(st, col_off, &sc->bar, val, col, nnz, ts, te, pol_stream);
             if (nxt.nr < 0) nxt = next_unit();
             // how the rows share the lanes, while the copy is on its way
             int32_t steps = 0;
@@ -504,7 +585,10 @@ __global__ void __launch_bounds__(P::kRowWarps * 32, 1)
                     const int32_t rs = inside(rp[k + lrow], ts, te);
                     const int32_t len = inside(rp[k + lrow + 1], rs, te) - rs;
                     const int32_t n = MULTI ? (len - sub + (1 << gs) - 1) >> gs : len;
-                    const int32_t nmax = (int32_t)__reduce_max_sync(FULL, (unsigned)n);
+                    // (of a single group: counted above)
+                    const int32_t nmax = jn == j + rows
+                                             ? steps
+                                             : (int32_t)__reduce_max_sync(FULL, (unsigned)n);
                     const int32_t nmin = (int32_t)__reduce_min_sync(FULL, (unsigned)n);
                     const int32_t first = rs - ts + off + sub;
                     // rows that start in a few banks only (lengths that are a
@@ -514,11 +598,11 @@ __global__ void __launch_bounds__(P::kRowWarps * 32, 1)
                         __reduce_or_sync(FULL, n > 0 ? 1u << (first & 31) : 0u);
                     A acc;
                     if (__popc(banks) <= 8 && nmax >= 8)
-                        acc = lane_dot<P, 4, MULTI ? 0 : 1, true>(
+                        acc = lane_dot<P, P::kLaneBatch, MULTI ? 0 : 1, true>(
                             sv + first, scol + first, x, n, nmin, nmax, 1 << gs,
                             n > 0 ? lrow % n : 0, pol_keep);
                     else
-                        acc = lane_dot<P, 4, MULTI ? 0 : 1, false>(
+                        acc = lane_dot<P, P::kLaneBatch, MULTI ? 0 : 1, false>(
                             sv + first, scol + first, x, n, nmin, nmax, 1 << gs, 0, pol_keep);
                     if (MULTI)
                         for (int d = 1; d < (1 << gs); d <<= 1)
@@ -593,12 +677,12 @@ struct FourRows {
 // lane 0's sum of piece w of row it.x (len entries) is in; the warp that
 // brings the row's last piece adds the pieces up, in a fixed order
 template <class P>
-__device__ __noinline__ void finish_piece(const RowArgs &a, uint32_t w, int2 it, int32_t len,
-                                          double sum)
+__device__ __noinline__ void finish_piece(const RowArgs &a, typename P::y_t *y, int32_t pl,
+                                          uint32_t w, int2 it, int32_t len, double sum)
 {
     using Y = typename P::y_t;
     const int lane = threadIdx.x & 31;
-    const int32_t n = (len + (1 << a.shape.piece) - 1) >> a.shape.piece;
+    const int32_t n = (len + (1 << pl) - 1) >> pl;
     const uint32_t first = w - (uint32_t)it.y;
     uint32_t seen = 0;
     if (lane == 0) {
@@ -614,12 +698,11 @@ __device__ __noinline__ void finish_piece(const RowArgs &a, uint32_t w, int2 it,
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) t += __shfl_xor_sync(FULL, t, d);
     if (lane == 0) {
-        Y *y = static_cast<Y *>(a.y);
-        y[it.x] = scaled_store_value(y, it.x, (Y)t, a.alpha, a.beta, a.axpby);
+        y[it.x] = row_value(a, y, it.x, (Y)t);
     }
 }
 
-template <class P, int UN, int BLOCKS>
+template <class P, int UN, int BLOCKS, bool BATCHED = false>
 __global__ void __launch_bounds__(kTailThreads, BLOCKS) rowtail_kernel(const RowArgs a)
 {
     using V = typename P::val_t;
@@ -637,12 +720,13 @@ __global__ void __launch_bounds__(kTailThreads, BLOCKS) rowtail_kernel(const Row
     const V *__restrict__ val = static_cast<const V *>(a.val);
     const X *__restrict__ x = static_cast<const X *>(a.x);
     const int32_t *__restrict__ col = a.col;
+    const int32_t *__restrict__ row_ptr = a.row_ptr;
     Y *y = static_cast<Y *>(a.y);
-    const int32_t m = a.m, nnz = a.nnz;
-    const int pl = a.shape.piece;
+    int32_t m = a.m, nnz = a.nnz;
+    int pl = a.shape.piece;
     const uint64_t pol = policy_evict_last();
     auto rp = [&](int32_t r) {
-        const int32_t p = __ldg(a.row_ptr + r);
+        const int32_t p = __ldg(row_ptr + r);
         return p < 0 ? 0 : (p > nnz ? nnz : p);
     };
     const uint32_t warps = gridDim.x * (kTailThreads / 32);
@@ -661,6 +745,17 @@ __global__ void __launch_bounds__(kTailThreads, BLOCKS) rowtail_kernel(const Row
         // long row: lane 0's
         const bool piece = w < np;
         const int2 it = piece ? a.pieces[w] : a.ranges[(w - np) / nsub];
+        if constexpr (BATCHED) {
+            const RowMat *mm = a.mats + (piece ? a.piece_mat[w] : a.range_mat[(w - np) / nsub]);
+            val = static_cast<const V *>(ldg_ptr(&mm->val));
+            x = static_cast<const X *>(ldg_ptr(&mm->x));
+            y = static_cast<Y *>(ldg_ptr(const_cast<void *const *>(&mm->y)));
+            col = ldg_ptr(&mm->col);
+            row_ptr = ldg_ptr(&mm->row_ptr);
+            m = __ldg(&mm->m);
+            nnz = __ldg(&mm->nnz);
+            pl = __ldg(&mm->packed) >> 16;
+        }
         const uint32_t sub = piece ? 0u : (w - np) & (nsub - 1);
         const bool in = piece ? lane == 0 : lane < it.y && it.x + lane < m;
         int32_t s = in ? rp(it.x + lane) : 0, e = in ? rp(it.x + lane + 1) : 0;
@@ -694,8 +789,7 @@ __global__ void __launch_bounds__(kTailThreads, BLOCKS) rowtail_kernel(const Row
                     }
                 }
                 if (isshort)
-                    y[it.x + lane] = scaled_store_value(y, it.x + lane, P::out(acc), a.alpha,
-                                                        a.beta, a.axpby);
+                    y[it.x + lane] = row_value(a, y, it.x + lane, P::out(acc));
             }
             todo = __ballot_sync(FULL, in && !isshort && row_len <= (1 << pl));
         }
@@ -765,10 +859,10 @@ __global__ void __launch_bounds__(kTailThreads, BLOCKS) rowtail_kernel(const Row
             for (; q < 4; ++q) r4.add(q, acc, lane);
             const A t = r4.sum(lane);
             if (piece) {
-                finish_piece<P>(a, w, it, __shfl_sync(FULL, row_len, 0), P::to_f64(t));
+                finish_piece<P>(a, y, pl, w, it, __shfl_sync(FULL, row_len, 0), P::to_f64(t));
             } else if ((lane & 7) == 0 && src >= 0) {
                 const int32_t r = it.x + src;
-                y[r] = scaled_store_value(y, r, P::out(t), a.alpha, a.beta, a.axpby);
+                y[r] = row_value(a, y, r, P::out(t));
             }
             q = 0;
             src = -1;
@@ -824,11 +918,11 @@ cudaError_t allow_smem(K kernel, int (&done)[64])
     return e;
 }
 
-template <class P, bool MULTI>
+template <class P, bool MULTI, bool BATCHED = false>
 int launch_rowblock(const Call &c, const RowArgs &a)
 {
     static int done[64] = {0};
-    cudaError_t e = allow_smem(rowblock_kernel<P, MULTI>, done);
+    cudaError_t e = allow_smem(rowblock_kernel<P, MULTI, BATCHED>, done);
     if (e != cudaSuccess) return record_cuda_error(e);
     // A gather that misses L1 holds one of its lines until it is served, so L1
     // has to be large enough for the gathers in flight: with all of shared
@@ -844,17 +938,17 @@ int launch_rowblock(const Call &c, const RowArgs &a)
     const unsigned grid = (unsigned)(a.nunits < sms ? a.nunits : sms);
     const int32_t need = (int32_t)((a.nunits + (int64_t)grid - 1) / grid);
     if (warps > need) warps = need;
-    e = launch_dependent(rowblock_kernel<P, MULTI>, grid, (unsigned)warps * 32,
+    e = launch_dependent(rowblock_kernel<P, MULTI, BATCHED>, grid, (unsigned)warps * 32,
                          (size_t)warps * (s.bytes + sizeof(RowScratch)), c.stream, a, s.bytes,
                          s.col_off);
     return e == cudaSuccess ? SSSPMV_OK : record_cuda_error(e);
 }
 
 // (r2) with at most one wave of blocks: a warp per listed range or piece
-template <class P, int UN, int BLOCKS>
+template <class P, int UN, int BLOCKS, bool BATCHED = false>
 int launch_rowtail(const Call &c, const RowArgs &a)
 {
-    auto k2 = rowtail_kernel<P, UN, BLOCKS>;
+    auto k2 = rowtail_kernel<P, UN, BLOCKS, BATCHED>;
     static int blocks[64] = {0};  // resident per SM
     int dev = 0;
     cudaGetDevice(&dev);
@@ -908,10 +1002,9 @@ int run_rowblock(const Call &c)
     a.max_pieces = (int32_t)rl.pieces;
     a.m = c.m;
     a.nnz = c.nnz;
-    // three quarters of the rows in units of several groups
-    const int32_t rows = 32 >> a.shape.gs, big_rows = rows << a.shape.us;
-    a.nbig = a.shape.us > 0 ? (int32_t)((int64_t)c.m * 3 / 4 / big_rows) : 0;
-    a.nunits = a.nbig + (int32_t)(((int64_t)c.m - (int64_t)a.nbig * big_rows + rows - 1) / rows);
+    const RowUnits units = row_units(c.m, a.shape);
+    a.nbig = units.nbig;
+    a.nunits = units.nunits;
     a.alpha = c.alpha;
     a.beta = c.beta;
     a.axpby = c.axpby;

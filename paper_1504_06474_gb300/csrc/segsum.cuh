@@ -37,6 +37,7 @@ struct F64 {
     static constexpr bool kEarlyLongScan = true;
     static constexpr int kShortRowWarps = 14;  // short rows: keep L1 for the gathers (measured)
     static constexpr int kRowWarps = 20;  // row blocks: warps per block (96 registers)
+    static constexpr int kLaneBatch = 4, kSplitBatch = 4;  // gathers in flight per lane
     // row blocks: a group of T entries whose longest lane takes n steps keeps
     // a lane per row (or G lanes) rather than an even split of its entries
     __device__ static __forceinline__ bool rows_even(int n, int T) { return n <= (T >> 5) + (T >> 6) + 8; }
@@ -102,9 +103,11 @@ struct CompF32Traits {
     static constexpr bool kEarlyLongScan = false;  // see F64
     static constexpr int kShortRowWarps = 16;  // short rows: keep L1 for the gathers (measured)
     static constexpr int kRowWarps = 24;  // 80 registers
+    // (eight or more in flight: more code and no faster)
+    static constexpr int kLaneBatch = 4, kSplitBatch = 4;
     __device__ static __forceinline__ bool rows_even(int n, int T)  // see F64
     {
-        return 16 * n <= (T >> 5) * 28 + 240;
+        return 16 * n <= (T >> 5) * 40 + 240;
     }
     using val_t = V;
     using x_t = float;

@@ -1,6 +1,7 @@
 // spmv_bf16.cu -- BF16-value instantiations: val in bfloat16, x and y in float,
 // compensated FP32 accumulation as in spmv_f32.cu.
 #include "launch.cuh"
+#include "rowblock.cuh"
 
 namespace ssspmv {
 
@@ -25,6 +26,7 @@ int bf16_resolve(Layout &l, int32_t S_opt)
 
 int bf16_run(Call &c)
 {
+    if (c.rows) return run_rowblock<BF16C>(c);
     switch (c.lay.W) {
 #define X(w) case w: return run_shape<BF16C, w>(c);
         SSSPMV_SHAPES(X)

@@ -1,6 +1,7 @@
 // spmv_f32.cu -- FP32 instantiations: val, x, y in float; each segment sum is an
 // unevaluated pair s + c updated by TwoProduct/TwoSum (compensated FP32).
 #include "launch.cuh"
+#include "rowblock.cuh"
 
 namespace ssspmv {
 
@@ -25,6 +26,7 @@ int f32_resolve(Layout &l, int32_t S_opt)
 
 int f32_run(Call &c)
 {
+    if (c.rows) return run_rowblock<F32C>(c);
     switch (c.lay.W) {
 #define X(w) case w: return run_shape<F32C, w>(c);
         SSSPMV_SHAPES(X)

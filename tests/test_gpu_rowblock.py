@@ -108,3 +108,50 @@ def test_f64_rounding(dev, kind):
     C.check(C.ssspmv_csr_f64(m, n, int(rp[-1]), rpd, cd, vd, xd, y), "csr")
     yref, s = oracle.spmv_dot2(rp, col, val, x)
     assert np.all(np.abs(y.cpu().numpy() - yref) <= 1e-13 * s)
+
+
+@pytest.mark.parametrize("prec", ["f32", "bf16"])
+@pytest.mark.parametrize("kind", KINDS)
+def test_reduced_precision_equals_the_row_loop(dev, kind, prec):
+    # every product and sum is an integer below 2^24: exact in FP32 too
+    from paper_1504_06474_gb300 import ssspmv as C
+    for m in (33, 1000, 9001):
+        if kind == "const1100" and m > 1000:
+            continue
+        rp, col, val, x = _matrix(kind, m, 517, seed=m + 1)
+        nnz, want = int(rp[-1]), oracle.spmv(rp, col, val, x)
+        vt = torch.float32 if prec == "f32" else torch.bfloat16
+        rpd, cd = _device(dev, (rp, col))
+        vd = torch.as_tensor(val, device=dev).to(vt)
+        xd = torch.as_tensor(x, device=dev).float()
+        fn = C.ssspmv_csr_f32 if prec == "f32" else C.ssspmv_csr_bf16f32
+        if prec == "bf16":
+            vd = vd.view(torch.int16)
+        y = torch.full((m,), float("nan"), dtype=torch.float32, device=dev)
+        C.check(fn(m, 517, nnz, rpd, cd, vd, xd, y), prec)
+        assert np.array_equal(y.cpu().numpy().astype(np.float64), want), (kind, m)
+
+
+def test_batch_of_every_kind(dev):
+    from paper_1504_06474_gb300 import ssspmv as C
+    keep, descs, wants, ys = [], [], [], []
+    for i, kind in enumerate(KINDS * 2):
+        m = (1, 33, 700, 5000)[i % 4]
+        rp, col, val, x = _matrix(kind, m, 517, seed=100 + i)
+        rpd, cd = _device(dev, (rp, col))
+        vd, xd = (torch.as_tensor(a, device=dev).float() for a in (val, x))
+        y = torch.full((m,), float("nan"), dtype=torch.float32, device=dev)
+        keep.append((rpd, cd, vd, xd))
+        descs.append((m, 517, int(rp[-1]), rpd, cd, vd, xd, y))
+        wants.append(oracle.spmv(rp, col, val, x))
+        ys.append(y)
+    total = sum(d[2] for d in descs)
+    desc = torch.frombuffer(bytearray(C.batch_descriptors(descs)), dtype=torch.uint8).to(dev)
+    ws = torch.full((C.ssspmv_batched_workspace_bytes(len(descs), total),), 255,
+                    dtype=torch.uint8, device=dev)
+    for _ in range(2):
+        C.check(C.ssspmv_csr_batched_f32(len(descs), desc, total, workspace=ws), "batched")
+        assert C.ssspmv_device_status(ws) == 0
+        for y, want in zip(ys, wants):
+            assert np.array_equal(y.cpu().numpy().astype(np.float64), want)
+            y.fill_(float("nan"))
