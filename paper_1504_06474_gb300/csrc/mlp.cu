@@ -13,7 +13,7 @@ namespace ssspmv {
 
 // ---------------------------------------------------------------------------
 // features: one pass over the row lengths, block partial sums into 64-bit
-// global counters, then one thread turns the counters into the 16 features
+// global counters, which the last block turns into the 16 features
 
 constexpr int kFeatThreads = 256;
 constexpr int kHistBins = 32;  // bin b: row length in [2^(b-1), 2^b), bin 0: empty
@@ -24,11 +24,11 @@ enum {
     FC_MAX,             // max len
     FC_EMPTY,           // empty rows
     FC_SHORT,           // rows with len <= 4
-    FC_HEAVY,           // rows with len >= 2 * mean (needs the mean: second pass)
+    FC_HEAVY,           // rows with len >= 2 * mean
     FC_LONGNNZ,         // entries in rows longer than 1024
     FC_JUMP,            // rows whose length differs from the previous row's by more than 2x
     FC_EMPTYRUN,        // empty rows followed by an empty row
-    FC_XNNZ,            // entries in rows of at least 32 * mean (second pass)
+    FC_XNNZ,            // entries in rows of at least 32 * mean
     FC_HIST,            // kHistBins counters
     FC_COUNT = FC_HIST + kHistBins
 };
@@ -39,108 +39,181 @@ __device__ __forceinline__ int len_bin(int32_t len)
                                                                   : kHistBins - 1);
 }
 
-// pass 1 (second == 0) or pass 2 (second == 1, the mean known)
+// All counters in one pass over row_ptr (the mean, and with it the thresholds
+// t2 = ceil(2 mean) and t32 = ceil(32 mean), is nnz / m and needs none), then
+// the last block to finish turns them into the features.  A warp takes 32 rows
+// at a time, one load per row; counts are ballots, and the histogram adds one
+// number per distinct bin of the 32 rows to the warp's own row of shared
+// memory (64-bit shared atomics per row, two passes and a single thread's FP64
+// divisions and logarithms at the end took 250 us of 2^21 rows; now 9).  The
+// upper half of FC_SHORT counts the blocks that are done.
 __global__ void __launch_bounds__(kFeatThreads)
-    feature_count_kernel(const int32_t *__restrict__ row_ptr, int32_t m, int32_t nnz, int second,
-                         unsigned long long *__restrict__ cnt)
+    feature_kernel(const int32_t *__restrict__ row_ptr, int32_t m, int32_t nnz, uint32_t t2,
+                   uint32_t t32, unsigned long long *__restrict__ cnt, float *__restrict__ f)
 {
+    constexpr int WARPS = kFeatThreads / 32;
     __shared__ unsigned long long s[FC_COUNT];
+    __shared__ uint32_t s_hist[WARPS][kHistBins];
+    __shared__ bool s_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < FC_COUNT; i += blockDim.x) s[i] = 0ull;
+    s_hist[warp][lane] = 0u;
     __syncthreads();
-    const double mean = m > 0 ? (double)nnz / (double)m : 0.0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long sum2 = 0, mx = 0, empty = 0, shrt = 0, heavy = 0, longnnz = 0, jump = 0,
-                       erun = 0, xnnz = 0;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m; r += stride) {
-        const int32_t a = __ldg(row_ptr + r), b = __ldg(row_ptr + r + 1);
-        const int32_t len = b - a;
-        if (!second) {
+    unsigned long long sum2 = 0, longnnz = 0, xnnz = 0;
+    uint32_t mx = 0, empty = 0, shrt = 0, heavy = 0, jump = 0, erun = 0;
+    const int64_t stride = (int64_t)gridDim.x * WARPS * 32;
+    constexpr int U = 4;  // chunks of 32 rows in flight
+    for (int64_t c = ((int64_t)blockIdx.x * WARPS + warp) * 32; c < m; c += U * stride) {
+        int32_t a[U], edge[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t r = c + u * stride + lane;
+            a[u] = r <= m ? __ldg(row_ptr + r) : 0;
+            // lane 0: the row before the chunk's; lane 31: the chunk's end
+            const int64_t q = lane == 0 ? r - 1 : r + 1;
+            edge[u] = ((lane == 0 && r > 0) || lane == 31) && q <= m ? __ldg(row_ptr + q) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (c + u * stride >= m) break;  // the same for the whole warp
+            const int64_t r = c + u * stride + lane;
+            const bool in = r < m;
+            int32_t b = __shfl_down_sync(FULL, a[u], 1);
+            if (lane == 31) b = edge[u];
+            int32_t before = __shfl_up_sync(FULL, a[u], 1);
+            if (lane == 0) before = edge[u];
+            const int32_t len = in ? b - a[u] : 0;
+            const int32_t p = a[u] - before;  // the previous row's length
+            const bool after = in && r > 0;
             sum2 += (unsigned long long)len * (unsigned long long)len;
-            mx = len > (int64_t)mx ? (unsigned long long)len : mx;
-            empty += len == 0;
-            shrt += len <= 4;
-            if (len > 1024) longnnz += (unsigned long long)len;
-            if (r > 0) {
-                const int32_t p = a - __ldg(row_ptr + r - 1);
-                jump += (len > 2 * p + 1) || (p > 2 * len + 1);
-                erun += (len == 0) && (p == 0);
-            }
-            atomicAdd(&s[FC_HIST + len_bin(len)], 1ull);
-        } else {
-            heavy += (double)len >= 2.0 * mean;
-            if ((double)len >= 32.0 * mean) xnnz += (unsigned long long)len;
+            mx = len > 0 && (uint32_t)len > mx ? (uint32_t)len : mx;
+            if (len > 1024) longnnz += (uint32_t)len;
+            if (in && len >= 0 && (uint32_t)len >= t32) xnnz += (uint32_t)len;
+            empty += __popc(__ballot_sync(FULL, in && len == 0));
+            shrt += __popc(__ballot_sync(FULL, in && len <= 4));
+            heavy += __popc(__ballot_sync(FULL, in && len >= 0 && (uint32_t)len >= t2));
+            jump += __popc(__ballot_sync(FULL, after && (len > 2 * p + 1 || p > 2 * len + 1)));
+            erun += __popc(__ballot_sync(FULL, after && len == 0 && p == 0));
+            const int bin = in ? len_bin(len) : kHistBins;
+            const unsigned same = __match_any_sync(FULL, bin);
+            if (in && lane == __ffs(same) - 1) s_hist[warp][bin] += __popc(same);
+            __syncwarp();
         }
     }
-    atomicAdd(&s[FC_SUM2], sum2);
-    atomicMax(&s[FC_MAX], mx);
-    atomicAdd(&s[FC_EMPTY], empty);
-    atomicAdd(&s[FC_SHORT], shrt);
-    atomicAdd(&s[FC_HEAVY], heavy);
-    atomicAdd(&s[FC_LONGNNZ], longnnz);
-    atomicAdd(&s[FC_JUMP], jump);
-    atomicAdd(&s[FC_EMPTYRUN], erun);
-    atomicAdd(&s[FC_XNNZ], xnnz);
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) {
+        sum2 += __shfl_xor_sync(FULL, sum2, d);
+        longnnz += __shfl_xor_sync(FULL, longnnz, d);
+        xnnz += __shfl_xor_sync(FULL, xnnz, d);
+    }
+    mx = __reduce_max_sync(FULL, mx);
+    if (lane == 0) {
+        atomicAdd(&s[FC_SUM2], sum2);
+        atomicMax(&s[FC_MAX], (unsigned long long)mx);
+        atomicAdd(&s[FC_EMPTY], (unsigned long long)empty);
+        atomicAdd(&s[FC_SHORT], (unsigned long long)shrt);
+        atomicAdd(&s[FC_HEAVY], (unsigned long long)heavy);
+        atomicAdd(&s[FC_LONGNNZ], longnnz);
+        atomicAdd(&s[FC_JUMP], (unsigned long long)jump);
+        atomicAdd(&s[FC_EMPTYRUN], (unsigned long long)erun);
+        atomicAdd(&s[FC_XNNZ], xnnz);
+    }
+    __syncthreads();
+    if (threadIdx.x < kHistBins) {
+        unsigned long long h = 0;
+        for (int w = 0; w < WARPS; ++w) h += s_hist[w][threadIdx.x];
+        s[FC_HIST + threadIdx.x] = h;
+    }
     __syncthreads();
     for (int i = threadIdx.x; i < FC_COUNT; i += blockDim.x) {
         if (i == FC_MAX) atomicMax(cnt + i, s[i]);
         else if (s[i]) atomicAdd(cnt + i, s[i]);
+        __threadfence();
     }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        s_last = (uint32_t)(atomicAdd(cnt + FC_SHORT, 1ull << 32) >> 32) == gridDim.x - 1u;
+    __syncthreads();
+    if (!s_last || warp != 0) return;
+    __threadfence();
+
+    // ---- the 16 features, one per lane; the FP64 steps they share (divisions,
+    // logarithms) are taken by all lanes together
+    auto count = [&](int i) {
+        unsigned long long v = __ldcg(cnt + i);
+        if (i == FC_SHORT) v &= 0xffffffffull;
+        return (double)v;
+    };
+    const double md = m > 0 ? (double)m : 1.0, nz = nnz > 0 ? (double)nnz : 1.0;
+    // percentiles of log2 length from the histogram: the first bin at which
+    // the count reaches q * m
+    unsigned long long cum = __ldcg(cnt + FC_HIST + lane);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned long long o = __shfl_up_sync(FULL, cum, d);
+        if (lane >= d) cum += o;
+    }
+    const double qs = lane == 9 ? 0.5 : (lane == 10 ? 0.9 : 0.99);
+    const double want = qs * md;
+    int pv = 0;
+    for (int k = 0; k < 3; ++k) {
+        const double w = __shfl_sync(FULL, want, 9 + k);
+        const unsigned hit = __ballot_sync(FULL, (double)cum >= w);
+        if (lane == 9 + k) pv = hit ? __ffs(hit) - 1 : 0;
+    }
+    // counts over rows or entries; lane 2: the mean, lane 3: the mean square
+    int which = FC_EMPTY;
+    if (lane == 3) which = FC_SUM2;
+    if (lane == 4) which = FC_MAX;
+    if (lane == 6) which = FC_SHORT;
+    if (lane == 7) which = FC_HEAVY;
+    if (lane == 8) which = FC_LONGNNZ;
+    if (lane == 12) which = FC_JUMP;
+    if (lane == 14) which = FC_EMPTYRUN;
+    if (lane == 15) which = FC_XNNZ;
+    const double c = count(which);
+    double v = (lane == 2 ? (double)nnz : c) / (lane == 8 || lane == 15 ? nz : md);
+    const double mean = __shfl_sync(FULL, v, 2);
+    if (lane == 3) {
+        const double var = v - mean * mean;
+        v = var > 0 ? sqrt(var) : 0.0;
+    }
+    if (lane == 13) v = 480.0;  // rows per 480-entry tile
+    if (lane == 3 || lane == 13) v /= lane == 3 ? mean + 1.0 : mean + 1e-9;
+    if (lane == 0) v = md;
+    if (lane == 1) v = (double)nnz;
+    if (lane == 4) v = c;
+    if (lane < 3 || lane == 4 || lane == 13) {
+        const double scale = lane == 1 ? 32.0 : (lane == 2 ? 8.0 : (lane == 13 ? 16.0 : 24.0));
+        v = log2(v + 1.0) / scale;
+    }
+    if (lane >= 9 && lane <= 11) v = (double)pv / 16.0;
+    if (lane < 16) f[lane] = (float)v;
 }
 
-// the 16 features, each of order one
-__global__ void feature_finish_kernel(const unsigned long long *__restrict__ cnt, int32_t m,
-                                      int32_t n, int32_t nnz, float *__restrict__ f)
+// the smallest row length at least k times the mean (as FP64 compares them)
+static uint32_t at_least(double k, double mean)
 {
-    if (threadIdx.x != 0) return;
-    const double md = m > 0 ? (double)m : 1.0;
-    const double mean = (double)nnz / md;
-    const double var = (double)cnt[FC_SUM2] / md - mean * mean;
-    const double sd = var > 0 ? sqrt(var) : 0.0;
-    const double nz = nnz > 0 ? (double)nnz : 1.0;
-    // histogram percentiles as log2 lengths
-    double q[3] = {0.5, 0.9, 0.99}, pv[3] = {0, 0, 0};
-    for (int k = 0; k < 3; ++k) {
-        double acc = 0.0;
-        for (int b = 0; b < kHistBins; ++b) {
-            acc += (double)cnt[FC_HIST + b];
-            if (acc >= q[k] * md) {
-                pv[k] = (double)b;
-                break;
-            }
-        }
-    }
-    f[0] = (float)(log2(md + 1.0) / 24.0);
-    f[1] = (float)(log2((double)nnz + 1.0) / 32.0);
-    f[2] = (float)(log2(mean + 1.0) / 8.0);
-    f[3] = (float)(sd / (mean + 1.0));
-    f[4] = (float)(log2((double)cnt[FC_MAX] + 1.0) / 24.0);
-    f[5] = (float)((double)cnt[FC_EMPTY] / md);
-    f[6] = (float)((double)cnt[FC_SHORT] / md);
-    f[7] = (float)((double)cnt[FC_HEAVY] / md);
-    f[8] = (float)((double)cnt[FC_LONGNNZ] / nz);
-    f[9] = (float)(pv[0] / 16.0);
-    f[10] = (float)(pv[1] / 16.0);
-    f[11] = (float)(pv[2] / 16.0);
-    f[12] = (float)((double)cnt[FC_JUMP] / md);
-    f[13] = (float)(log2(480.0 / (mean + 1e-9) + 1.0) / 16.0);  // rows per 480-entry tile
-    f[14] = (float)((double)cnt[FC_EMPTYRUN] / md);
-    f[15] = (float)((double)cnt[FC_XNNZ] / nz);
-    (void)n;
+    const double t = std::ceil(k * mean);
+    return t >= 4294967295.0 ? 0xffffffffu : (uint32_t)t;
 }
 
 int run_features(const int32_t *row_ptr, int32_t m, int32_t n, int32_t nnz, float *out,
                  void *scratch, cudaStream_t s)
 {
+    (void)n;
     unsigned long long *cnt = static_cast<unsigned long long *>(scratch);
     cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * FC_COUNT, s);
     if (e != cudaSuccess) return record_cuda_error(e);
-    int64_t blocks = ((int64_t)m + kFeatThreads - 1) / kFeatThreads;
-    const int64_t cap = 8LL * device_sm_count();
+    // four chunks of 32 rows per warp, four blocks per SM at most (the blocks
+    // meet in the counters' atomics)
+    int64_t blocks = ((int64_t)m + 4 * kFeatThreads - 1) / (4 * kFeatThreads);
+    const int64_t cap = 4LL * device_sm_count();
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    for (int pass = 0; pass < 2; ++pass)
-        feature_count_kernel<<<(unsigned)blocks, kFeatThreads, 0, s>>>(row_ptr, m, nnz, pass, cnt);
-    feature_finish_kernel<<<1, 32, 0, s>>>(cnt, m, n, nnz, out);
+    const double mean = m > 0 ? (double)nnz / (double)m : 0.0;
+    feature_kernel<<<(unsigned)blocks, kFeatThreads, 0, s>>>(row_ptr, m, nnz, at_least(2.0, mean),
+                                                            at_least(32.0, mean), cnt, out);
     e = cudaGetLastError();
     if (e != cudaSuccess) return record_cuda_error(e);
     return SSSPMV_OK;
