@@ -302,6 +302,8 @@ __global__ void __launch_bounds__(kMlpThreads)
                 float wd, int t)
 {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    grid_dep_wait();  // the gradient comes from the kernel before
+    grid_dep_trigger();
     if (k >= n) return;
     const float gk = g[k] + wd * p[k];
     const float a = b1 * m1[k] + (1.0f - b1) * gk;
@@ -328,6 +330,270 @@ __global__ void argmin_kernel(const float *__restrict__ out, int B, int K, int32
         }
     }
     cls[b] = best;
+}
+
+// ---------------------------------------------------------------------------
+// The selector's own sizes (64 units in both hidden layers, up to 32 features
+// and classes) in one kernel: a block takes kMlpTile samples through all
+// layers with every weight and activation in shared memory, and for training
+// back again, leaving its samples' share of the weight gradients in `parts`;
+// mlp_reduce_kernel adds the blocks' shares in order.  One layer per launch
+// and one thread per weight over the whole batch took 960 us for a training
+// step on 2,000 samples, nearly all of it the weight gradients' serial sums;
+// this takes 20.
+
+constexpr int kMlpH = 64, kMlpMaxF = 32, kMlpMaxK = 32, kMlpTile = 16;
+constexpr int kMlpLd = kMlpH + 4;  // rows of 64 a bank group apart, 16-byte aligned
+
+struct MlpSmem {
+    float W1t[kMlpMaxF][kMlpLd];  // W1t[i][o] = W1[o][i]
+    float W2t[kMlpH][kMlpLd];
+    float W2[kMlpH][kMlpLd];
+    float W3[kMlpMaxK][kMlpLd];
+    float b1[kMlpH], b2[kMlpH], b3[kMlpMaxK];
+    float X[kMlpTile][kMlpMaxF];
+    float a1[kMlpTile][kMlpLd], a2[kMlpTile][kMlpLd];
+    float g2[kMlpTile][kMlpLd], g1[kMlpTile][kMlpLd];
+    float o3[kMlpTile][kMlpMaxK], g3[kMlpTile][kMlpMaxK];
+};
+
+struct MlpArgs {
+    const float *params, *X;
+    float *out, *out2;     // predictions (out2 nullable)
+    int32_t *cls;          // nullable: the least prediction's class
+    const float *target;   // training: nullable otherwise
+    float *parts;          // training: [blocks][count + 1], the last the loss
+    float inv_count;
+    int32_t B, F, K, count;
+};
+
+// acc[q] += W[i][o] * in[b + 4 q][i] over i < n in order (n a multiple of 4)
+__device__ __forceinline__ void mlp_dot4(float (&acc)[4], const float (*W)[kMlpLd], int o,
+                                         const float *in, int ld, int n)
+{
+    for (int i = 0; i < n; i += 4) {
+        const float w0 = W[i][o], w1 = W[i + 1][o], w2 = W[i + 2][o], w3 = W[i + 3][o];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 v = *reinterpret_cast<const float4 *>(in + 4 * q * ld + i);
+            acc[q] = fmaf(w0, v.x, acc[q]);
+            acc[q] = fmaf(w1, v.y, acc[q]);
+            acc[q] = fmaf(w2, v.z, acc[q]);
+            acc[q] = fmaf(w3, v.w, acc[q]);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kMlpThreads) mlp_kernel(const MlpArgs a)
+{
+    extern __shared__ __align__(16) unsigned char mlp_smem[];
+    __shared__ float s_loss[kMlpThreads / 32];
+    MlpSmem &s = *reinterpret_cast<MlpSmem *>(mlp_smem);
+    constexpr int H = kMlpH;
+    const int t = threadIdx.x, F = a.F, K = a.K;
+    const float *W1 = a.params, *b1 = W1 + H * F, *W2 = b1 + H, *b2 = W2 + H * H, *W3 = b2 + H,
+                *b3 = W3 + K * H;
+    grid_dep_wait();  // the parameters may come from the kernel before
+    grid_dep_trigger();
+    for (int k = t; k < H * F; k += kMlpThreads) s.W1t[k % F][k / F] = __ldg(W1 + k);
+    for (int k = t; k < H * H; k += kMlpThreads) {
+        const float w = __ldg(W2 + k);
+        s.W2[k / H][k % H] = w;
+        s.W2t[k % H][k / H] = w;
+    }
+    for (int k = t; k < K * H; k += kMlpThreads) s.W3[k / H][k % H] = __ldg(W3 + k);
+    if (t < H) {
+        s.b1[t] = __ldg(b1 + t);
+        s.b2[t] = __ldg(b2 + t);
+    }
+    if (t < K) s.b3[t] = __ldg(b3 + t);
+    // tiles of samples (training: more than one where the scratch holds the
+    // shares of fewer blocks than there are tiles)
+    for (int b0 = blockIdx.x * kMlpTile; b0 < a.B; b0 += gridDim.x * kMlpTile) {
+        const bool first = b0 == (int)blockIdx.x * kMlpTile;
+        auto add = [&](float *at, float v) { *at = first ? v : *at + v; };
+        __syncthreads();  // the tile before is done with
+        for (int k = t; k < kMlpTile * F; k += kMlpThreads)
+            s.X[k / F][k % F] = b0 + k / F < a.B ? __ldg(a.X + (int64_t)b0 * F + k) : 0.0f;
+        __syncthreads();
+        // hidden layers: a thread takes one unit of samples sb, sb + 4, ..
+        const int o = t % H, sb = t / H;
+        float acc[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = s.b1[o];
+        mlp_dot4(acc, s.W1t, o, s.X[sb], kMlpMaxF, F);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s.a1[sb + 4 * q][o] = fmaxf(acc[q], 0.0f);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = s.b2[o];
+        mlp_dot4(acc, s.W2t, o, s.a1[sb], kMlpLd, H);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s.a2[sb + 4 * q][o] = fmaxf(acc[q], 0.0f);
+        __syncthreads();
+        float loss = 0.0f;
+        for (int k = t; k < kMlpTile * K; k += kMlpThreads) {
+            const int b = k / K, c = k % K;
+            float v = s.b3[c];
+            for (int i = 0; i < H; ++i) v = fmaf(s.W3[c][i], s.a2[b][i], v);
+            s.o3[b][c] = v;
+            float g = 0.0f;
+            if (b0 + b < a.B) {
+                const int64_t at = (int64_t)(b0 + b) * K + c;
+                if (a.out) a.out[at] = v;
+                if (a.out2) a.out2[at] = v;
+                if (a.target) {
+                    // a NaN target (a class not measured) counts as no error
+                    const float y = __ldg(a.target + at);
+                    const float d = (y == y) ? v - y : 0.0f;
+                    g = 2.0f * d * a.inv_count;
+                    loss += d * d * a.inv_count;
+                }
+            }
+            s.g3[b][c] = g;
+        }
+        if (a.cls) {
+            __syncthreads();
+            if (t < kMlpTile && b0 + t < a.B) {
+                int best = 0;
+                for (int c = 1; c < K; ++c)
+                    if (s.o3[t][c] < s.o3[t][best]) best = c;
+                a.cls[b0 + t] = best;
+            }
+        }
+        if (!a.target) continue;
+        float *part = a.parts + (int64_t)blockIdx.x * (a.count + 1);
+        float *dW1 = part, *db1 = dW1 + H * F, *dW2 = db1 + H, *db2 = dW2 + H * H, *dW3 = db2 + H,
+              *db3 = dW3 + K * H;
+        #pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) loss += __shfl_xor_sync(FULL, loss, d);
+        if ((t & 31) == 0) s_loss[t >> 5] = loss;
+        __syncthreads();
+        if (t == 0) {
+            float l = 0.0f;
+            for (int w = 0; w < kMlpThreads / 32; ++w) l += s_loss[w];
+            add(part + a.count, l);
+        }
+        // back through the output layer
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = 0.0f;
+        for (int c = 0; c < K; ++c) {
+            const float w = s.W3[c][o];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[q] = fmaf(w, s.g3[sb + 4 * q][c], acc[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            s.g2[sb + 4 * q][o] = s.a2[sb + 4 * q][o] > 0.0f ? acc[q] : 0.0f;
+        for (int k = t; k < K * H; k += kMlpThreads) {
+            const int c = k / H, i = k % H;
+            float v = 0.0f;
+#pragma unroll
+            for (int b = 0; b < kMlpTile; ++b) v = fmaf(s.g3[b][c], s.a2[b][i], v);
+            add(dW3 + k, v);
+        }
+        if (t < K) {
+            float v = 0.0f;
+            for (int b = 0; b < kMlpTile; ++b) v += s.g3[b][t];
+            add(db3 + t, v);
+        }
+        __syncthreads();
+        // and through the second hidden layer
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = 0.0f;
+        mlp_dot4(acc, s.W2, o, s.g2[sb], kMlpLd, H);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            s.g1[sb + 4 * q][o] = s.a1[sb + 4 * q][o] > 0.0f ? acc[q] : 0.0f;
+        {
+            // dW2: a thread takes 4 x 4 weights
+            const int o4 = (t / 16) * 4, i4 = (t % 16) * 4;
+            float w[4][4] = {};
+#pragma unroll
+            for (int b = 0; b < kMlpTile; ++b) {
+                const float4 g = *reinterpret_cast<const float4 *>(&s.g2[b][o4]);
+                const float4 v = *reinterpret_cast<const float4 *>(&s.a1[b][i4]);
+                const float gg[4] = {g.x, g.y, g.z, g.w}, vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) w[p][q] = fmaf(gg[p], vv[q], w[p][q]);
+            }
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) add(dW2 + (o4 + p) * H + i4 + q, w[p][q]);
+        }
+        if (t < H) {
+            float v = 0.0f;
+            for (int b = 0; b < kMlpTile; ++b) v += s.g2[b][t];
+            add(db2 + t, v);
+        }
+        __syncthreads();
+        for (int k = t; k < H * F; k += kMlpThreads) {
+            const int u = k / F, i = k % F;
+            float v = 0.0f;
+#pragma unroll
+            for (int b = 0; b < kMlpTile; ++b) v = fmaf(s.g1[b][u], s.X[b][i], v);
+            add(dW1 + k, v);
+        }
+        if (t < H) {
+            float v = 0.0f;
+            for (int b = 0; b < kMlpTile; ++b) v += s.g1[b][t];
+            add(db1 + t, v);
+        }
+    }
+}
+
+// grad[k] = the blocks' shares of weight k, added in order; the last one the loss
+__global__ void __launch_bounds__(kMlpThreads)
+    mlp_reduce_kernel(const float *__restrict__ parts, int32_t blocks, int32_t count,
+                      float *__restrict__ grad, float *__restrict__ loss)
+{
+    // 32 weights per warp row, eight rows of the block each an eighth of the
+    // blocks; their sums are joined in order
+    __shared__ float s_sum[kMlpThreads / 32][32];
+    grid_dep_wait();
+    grid_dep_trigger();
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    constexpr int ROWS = kMlpThreads / 32;
+    const int32_t k = blockIdx.x * 32 + lane;
+    const int32_t per = (blocks + ROWS - 1) / ROWS;
+    const int32_t lo = row * per, hi = lo + per < blocks ? lo + per : blocks;
+    float v = 0.0f;
+    if (k <= count) {
+#pragma unroll 8
+        for (int32_t b = lo; b < hi; ++b) v += __ldcg(parts + (int64_t)b * (count + 1) + k);
+    }
+    s_sum[row][lane] = v;
+    __syncthreads();
+    if (row != 0 || k > count) return;
+    v = 0.0f;
+    for (int r = 0; r < ROWS; ++r) v += s_sum[r][lane];
+    if (k < count) grad[k] = v;
+    else if (loss) *loss = v;
+}
+
+// whether the one-kernel path takes these sizes
+static bool mlp_fused(int32_t F, int32_t H1, int32_t H2, int32_t K)
+{
+    return H1 == kMlpH && H2 == kMlpH && F <= kMlpMaxF && F % 4 == 0 && K <= kMlpMaxK;
+}
+
+static int64_t mlp_tiles(int32_t B) { return ((int64_t)B + kMlpTile - 1) / kMlpTile; }
+
+static cudaError_t launch_mlp(const MlpArgs &a, int64_t blocks, cudaStream_t s)
+{
+    static int done[64] = {0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || !done[dev]) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            mlp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpSmem));
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) done[dev] = 1;
+    }
+    return launch_dependent(mlp_kernel, (unsigned)blocks, kMlpThreads, sizeof(MlpSmem), s, a);
 }
 
 static unsigned blocks_for(int64_t n) { return (unsigned)((n + kMlpThreads - 1) / kMlpThreads); }
@@ -366,6 +632,18 @@ size_t ssspmv_mlp_scratch_floats(int32_t B, int32_t F, int32_t H1, int32_t H2, i
     return (size_t)B * (2 * H1 + 2 * H2 + 2 * K + H2 + H1) + 1;
 }
 
+static MlpArgs mlp_args(const float *params, const float *X, int32_t B, int32_t F, int32_t K)
+{
+    MlpArgs a = {};
+    a.params = params;
+    a.X = X;
+    a.B = B;
+    a.F = F;
+    a.K = K;
+    a.count = (int32_t)mlp_param_count(F, kMlpH, kMlpH, K);
+    return a;
+}
+
 static int mlp_forward_impl(const float *params, const float *X, int32_t B, int32_t F, int32_t H1,
                             int32_t H2, int32_t K, float *scratch, cudaStream_t s)
 {
@@ -391,6 +669,13 @@ int ssspmv_mlp_forward(const float *params, const float *X, int32_t B, int32_t F
     if (!params || !X || !scratch || B <= 0 || F <= 0 || H1 <= 0 || H2 <= 0 || K <= 0)
         return SSSPMV_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (mlp_fused(F, H1, H2, K)) {
+        MlpArgs a = mlp_args(params, X, B, F, K);
+        a.out = scratch + (int64_t)B * (2 * H1 + 2 * H2);
+        a.out2 = out;
+        const cudaError_t e = launch_mlp(a, mlp_tiles(B), s);
+        return e == cudaSuccess ? SSSPMV_OK : record_cuda_error(e);
+    }
     int rc = mlp_forward_impl(params, X, B, F, H1, H2, K, scratch, s);
     if (rc) return rc;
     if (out) {
@@ -410,6 +695,23 @@ int ssspmv_mlp_backward(const float *params, const float *X, const float *target
         H2 <= 0 || K <= 0)
         return SSSPMV_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // a block per tile of samples, or as many as the scratch holds the shares of
+    int64_t blocks = mlp_tiles(B);
+    const int64_t room = (int64_t)(ssspmv_mlp_scratch_floats(B, F, H1, H2, K) /
+                                   (size_t)(mlp_param_count(F, H1, H2, K) + 1));
+    if (blocks > room) blocks = room;
+    if (mlp_fused(F, H1, H2, K) && blocks > 0) {
+        MlpArgs a = mlp_args(params, X, B, F, K);
+        a.target = target;
+        a.parts = scratch;
+        a.inv_count = 1.0f / (float)((int64_t)B * K);
+        cudaError_t e = launch_mlp(a, blocks, s);
+        if (e == cudaSuccess)
+            e = launch_dependent(mlp_reduce_kernel, (unsigned)((a.count + 1 + 31) / 32),
+                                 kMlpThreads, 0, s, (const float *)scratch, (int32_t)blocks,
+                                 a.count, grad, loss);
+        return e == cudaSuccess ? SSSPMV_OK : record_cuda_error(e);
+    }
     int rc = mlp_forward_impl(params, X, B, F, H1, H2, K, scratch, s);
     if (rc) return rc;
     const float *W2 = params + (int64_t)H1 * F + H1;
@@ -453,9 +755,8 @@ int ssspmv_mlp_adam(float *params, const float *grad, float *m1, float *m2, int6
 {
     if (!params || !grad || !m1 || !m2 || n <= 0 || step < 1) return SSSPMV_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    adam_kernel<<<blocks_for(n), kMlpThreads, 0, s>>>(params, grad, m1, m2, n, lr, beta1, beta2,
-                                                     eps, weight_decay, step);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_dependent(adam_kernel, blocks_for(n), kMlpThreads, 0, s, params, grad,
+                                     m1, m2, n, lr, beta1, beta2, eps, weight_decay, step);
     return e == cudaSuccess ? SSSPMV_OK : record_cuda_error(e);
 }
 
@@ -464,6 +765,13 @@ int ssspmv_mlp_select(const float *params, const float *X, int32_t B, int32_t F,
 {
     if (!cls) return SSSPMV_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (params && X && scratch && B > 0 && F > 0 && K > 0 && mlp_fused(F, H1, H2, K)) {
+        MlpArgs a = mlp_args(params, X, B, F, K);
+        a.out = scratch + (int64_t)B * (2 * H1 + 2 * H2);
+        a.cls = cls;
+        const cudaError_t e = launch_mlp(a, mlp_tiles(B), s);
+        return e == cudaSuccess ? SSSPMV_OK : record_cuda_error(e);
+    }
     int rc = ssspmv_mlp_forward(params, X, B, F, H1, H2, K, scratch, nullptr, stream);
     if (rc) return rc;
     const float *out = scratch + (int64_t)B * (2 * H1 + 2 * H2);
