@@ -127,23 +127,44 @@ def _ptr(a):
     if isinstance(a, int):
         return a
     if hasattr(a, "data_ptr"):
-        if a.numel() and not a.is_contiguous():
+        if not a.numel():
+            return None
+        if not a.is_contiguous():
             raise ValueError("tensor must be contiguous")
-        return a.data_ptr() if a.numel() else None
+        return a.data_ptr()
     if hasattr(a, "ctypes"):  # numpy array (host)
         return a.ctypes.data if a.size else None
     raise TypeError("cannot take the address of %r" % type(a))
 
 
-def _stream(s):
-    if s is None:
+_current = None  # () -> raw handle of the current torch stream, once CUDA is up
+
+
+def _current_stream():
+    """The current torch stream's handle.  The stream object that
+    torch.cuda.current_stream() makes for every call cost 3.9 us of the 12.5 us
+    a small product took on the host; the handle alone takes 0.3."""
+    global _current
+    if _current is None:
         try:
             import torch
-            if torch.cuda.is_available():
-                return torch.cuda.current_stream().cuda_stream
         except ImportError:
-            pass
-        return None
+            return None
+        if not torch.cuda.is_available():
+            return None
+        torch.cuda.init()
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        dev = getattr(torch._C, "_cuda_getDevice", None)
+        if raw is not None and dev is not None:
+            _current = lambda: raw(dev())  # noqa: E731
+        else:
+            _current = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
+    return _current()
+
+
+def _stream(s):
+    if s is None:
+        return _current_stream()
     if isinstance(s, int):
         return s
     return s.cuda_stream
