@@ -39,17 +39,25 @@ __device__ __forceinline__ int len_bin(int32_t len)
                                                                   : kHistBins - 1);
 }
 
+// the features that m and nnz alone decide
+struct HostFeatures {
+    double mean;
+    float f0, f1, f2, f13;
+};
+
 // All counters in one pass over row_ptr (the mean, and with it the thresholds
 // t2 = ceil(2 mean) and t32 = ceil(32 mean), is nnz / m and needs none), then
 // the last block to finish turns them into the features.  A warp takes 32 rows
-// at a time, one load per row; counts are ballots, and the histogram adds one
-// number per distinct bin of the 32 rows to the warp's own row of shared
-// memory (64-bit shared atomics per row, two passes and a single thread's FP64
-// divisions and logarithms at the end took 250 us of 2^21 rows; now 9).  The
-// upper half of FC_SHORT counts the blocks that are done.
+// at a time, one load per row; its bound is instruction issue, so each thread
+// keeps its own counts, and each warp its own histogram in shared memory.
+// (64-bit shared atomics per row, two passes and a single thread's FP64
+// divisions and logarithms at the end took 250 us of 2^21 rows; this takes 16,
+// 10 of them whatever the size.)  The upper half of FC_SHORT counts the blocks
+// that are done.
 __global__ void __launch_bounds__(kFeatThreads)
     feature_kernel(const int32_t *__restrict__ row_ptr, int32_t m, int32_t nnz, uint32_t t2,
-                   uint32_t t32, unsigned long long *__restrict__ cnt, float *__restrict__ f)
+                   uint32_t t32, const HostFeatures host, unsigned long long *__restrict__ cnt,
+                   float *__restrict__ f)
 {
     constexpr int WARPS = kFeatThreads / 32;
     __shared__ unsigned long long s[FC_COUNT];
@@ -60,44 +68,43 @@ __global__ void __launch_bounds__(kFeatThreads)
     s_hist[warp][lane] = 0u;
     __syncthreads();
     unsigned long long sum2 = 0, longnnz = 0, xnnz = 0;
-    uint32_t mx = 0, empty = 0, shrt = 0, heavy = 0, jump = 0, erun = 0;
-    const int64_t stride = (int64_t)gridDim.x * WARPS * 32;
+    int32_t mx = 0;
+    uint32_t empty = 0, shrt = 0, heavy = 0, jump = 0, erun = 0;
+    // (indices stay below 2^32: m is below 2^31, and so are U strides)
+    const uint32_t stride = gridDim.x * WARPS * 32u, rows = (uint32_t)m;
     constexpr int U = 4;  // chunks of 32 rows in flight
-    for (int64_t c = ((int64_t)blockIdx.x * WARPS + warp) * 32; c < m; c += U * stride) {
+    for (uint32_t c = (blockIdx.x * WARPS + warp) * 32u; c < rows; c += U * stride) {
         int32_t a[U], edge[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t r = c + u * stride + lane;
-            a[u] = r <= m ? __ldg(row_ptr + r) : 0;
+            const uint32_t r = c + u * stride + lane;
+            a[u] = edge[u] = 0;
+            if (r <= rows) a[u] = __ldg(row_ptr + r);
             // lane 0: the row before the chunk's; lane 31: the chunk's end
-            const int64_t q = lane == 0 ? r - 1 : r + 1;
-            edge[u] = ((lane == 0 && r > 0) || lane == 31) && q <= m ? __ldg(row_ptr + q) : 0;
+            if (lane == 0 && r > 0 && r <= rows) edge[u] = __ldg(row_ptr + r - 1);
+            if (lane == 31 && r < rows) edge[u] = __ldg(row_ptr + r + 1);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (c + u * stride >= m) break;  // the same for the whole warp
-            const int64_t r = c + u * stride + lane;
-            const bool in = r < m;
+            const uint32_t r = c + u * stride + lane;
             int32_t b = __shfl_down_sync(FULL, a[u], 1);
-            if (lane == 31) b = edge[u];
             int32_t before = __shfl_up_sync(FULL, a[u], 1);
+            if (lane == 31) b = edge[u];
             if (lane == 0) before = edge[u];
-            const int32_t len = in ? b - a[u] : 0;
-            const int32_t p = a[u] - before;  // the previous row's length
-            const bool after = in && r > 0;
-            sum2 += (unsigned long long)len * (unsigned long long)len;
-            mx = len > 0 && (uint32_t)len > mx ? (uint32_t)len : mx;
+            if (r >= rows) continue;
+            const int32_t len = b - a[u], p = a[u] - before;  // p: the previous row's length
+            sum2 += (unsigned long long)(uint32_t)len * (uint32_t)len;
+            mx = max(mx, len);
             if (len > 1024) longnnz += (uint32_t)len;
-            if (in && len >= 0 && (uint32_t)len >= t32) xnnz += (uint32_t)len;
-            empty += __popc(__ballot_sync(FULL, in && len == 0));
-            shrt += __popc(__ballot_sync(FULL, in && len <= 4));
-            heavy += __popc(__ballot_sync(FULL, in && len >= 0 && (uint32_t)len >= t2));
-            jump += __popc(__ballot_sync(FULL, after && (len > 2 * p + 1 || p > 2 * len + 1)));
-            erun += __popc(__ballot_sync(FULL, after && len == 0 && p == 0));
-            const int bin = in ? len_bin(len) : kHistBins;
-            const unsigned same = __match_any_sync(FULL, bin);
-            if (in && lane == __ffs(same) - 1) s_hist[warp][bin] += __popc(same);
-            __syncwarp();
+            if ((uint32_t)len >= t32) xnnz += (uint32_t)len;
+            if (len == 0) ++empty;
+            if (len <= 4) ++shrt;
+            if ((uint32_t)len >= t2) ++heavy;
+            if (r > 0) {
+                if (len > 2 * p + 1 || p > 2 * len + 1) ++jump;
+                if (len == 0 && p == 0) ++erun;
+            }
+            atomicAdd(&s_hist[warp][len_bin(len)], 1u);
         }
     }
 #pragma unroll
@@ -107,6 +114,11 @@ __global__ void __launch_bounds__(kFeatThreads)
         xnnz += __shfl_xor_sync(FULL, xnnz, d);
     }
     mx = __reduce_max_sync(FULL, mx);
+    empty = __reduce_add_sync(FULL, empty);
+    shrt = __reduce_add_sync(FULL, shrt);
+    heavy = __reduce_add_sync(FULL, heavy);
+    jump = __reduce_add_sync(FULL, jump);
+    erun = __reduce_add_sync(FULL, erun);
     if (lane == 0) {
         atomicAdd(&s[FC_SUM2], sum2);
         atomicMax(&s[FC_MAX], (unsigned long long)mx);
@@ -134,61 +146,53 @@ __global__ void __launch_bounds__(kFeatThreads)
     if (threadIdx.x == 0)
         s_last = (uint32_t)(atomicAdd(cnt + FC_SHORT, 1ull << 32) >> 32) == gridDim.x - 1u;
     __syncthreads();
-    if (!s_last || warp != 0) return;
+    if (!s_last || warp > 2) return;
     __threadfence();
 
-    // ---- the 16 features, one per lane; the FP64 steps they share (divisions,
-    // logarithms) are taken by all lanes together
-    auto count = [&](int i) {
-        unsigned long long v = __ldcg(cnt + i);
-        if (i == FC_SHORT) v &= 0xffffffffull;
-        return (double)v;
-    };
+    // ---- the features.  A lone warp's FP64 instructions are 65 cycles apart, so
+    // what depends on m and nnz alone comes from the host, and the rest goes by
+    // three warps: ratios (one division for all lanes), the logarithm, the
+    // percentiles
     const double md = m > 0 ? (double)m : 1.0, nz = nnz > 0 ? (double)nnz : 1.0;
-    // percentiles of log2 length from the histogram: the first bin at which
-    // the count reaches q * m
-    unsigned long long cum = __ldcg(cnt + FC_HIST + lane);
+    if (warp == 0) {
+        int which = FC_EMPTY;  // lane 5
+        if (lane == 3) which = FC_SUM2;
+        if (lane == 6) which = FC_SHORT;
+        if (lane == 7) which = FC_HEAVY;
+        if (lane == 8) which = FC_LONGNNZ;
+        if (lane == 12) which = FC_JUMP;
+        if (lane == 14) which = FC_EMPTYRUN;
+        if (lane == 15) which = FC_XNNZ;
+        unsigned long long c = __ldcg(cnt + which);
+        if (lane == 6) c &= 0xffffffffull;
+        double v = (double)c / (lane == 8 || lane == 15 ? nz : md);
+        if (lane == 3) {
+            const double var = v - host.mean * host.mean;
+            v = (var > 0 ? sqrt(var) : 0.0) / (host.mean + 1.0);
+        }
+        if (lane == 3 || (lane >= 5 && lane <= 8) || lane == 12 || lane == 14 || lane == 15)
+            f[lane] = (float)v;
+    } else if (warp == 1) {
+        if (lane == 0) f[0] = host.f0;
+        if (lane == 1) f[1] = host.f1;
+        if (lane == 2) f[2] = host.f2;
+        if (lane == 13) f[13] = host.f13;
+        if (lane == 4) f[4] = (float)(log2((double)__ldcg(cnt + FC_MAX) + 1.0) / 24.0);
+    } else {
+        // the first bin of the histogram at which the count reaches q * m
+        unsigned long long cum = __ldcg(cnt + FC_HIST + lane);
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned long long o = __shfl_up_sync(FULL, cum, d);
-        if (lane >= d) cum += o;
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned long long o = __shfl_up_sync(FULL, cum, d);
+            if (lane >= d) cum += o;
+        }
+        const double qs = lane == 9 ? 0.5 : (lane == 10 ? 0.9 : 0.99);
+        const double want = qs * md, have = (double)cum;
+        for (int k = 9; k < 12; ++k) {
+            const unsigned hit = __ballot_sync(FULL, have >= __shfl_sync(FULL, want, k));
+            if (lane == k) f[k] = (float)(hit ? __ffs(hit) - 1 : 0) / 16.0f;
+        }
     }
-    const double qs = lane == 9 ? 0.5 : (lane == 10 ? 0.9 : 0.99);
-    const double want = qs * md;
-    int pv = 0;
-    for (int k = 0; k < 3; ++k) {
-        const double w = __shfl_sync(FULL, want, 9 + k);
-        const unsigned hit = __ballot_sync(FULL, (double)cum >= w);
-        if (lane == 9 + k) pv = hit ? __ffs(hit) - 1 : 0;
-    }
-    // counts over rows or entries; lane 2: the mean, lane 3: the mean square
-    int which = FC_EMPTY;
-    if (lane == 3) which = FC_SUM2;
-    if (lane == 4) which = FC_MAX;
-    if (lane == 6) which = FC_SHORT;
-    if (lane == 7) which = FC_HEAVY;
-    if (lane == 8) which = FC_LONGNNZ;
-    if (lane == 12) which = FC_JUMP;
-    if (lane == 14) which = FC_EMPTYRUN;
-    if (lane == 15) which = FC_XNNZ;
-    const double c = count(which);
-    double v = (lane == 2 ? (double)nnz : c) / (lane == 8 || lane == 15 ? nz : md);
-    const double mean = __shfl_sync(FULL, v, 2);
-    if (lane == 3) {
-        const double var = v - mean * mean;
-        v = var > 0 ? sqrt(var) : 0.0;
-    }
-    if (lane == 13) v = 480.0;  // rows per 480-entry tile
-    if (lane == 3 || lane == 13) v /= lane == 3 ? mean + 1.0 : mean + 1e-9;
-    if (lane == 0) v = md;
-    if (lane == 1) v = (double)nnz;
-    if (lane == 4) v = c;
-    if (lane < 3 || lane == 4 || lane == 13) {
-        const double scale = lane == 1 ? 32.0 : (lane == 2 ? 8.0 : (lane == 13 ? 16.0 : 24.0));
-        v = log2(v + 1.0) / scale;
-    }
-    if (lane >= 9 && lane <= 11) v = (double)pv / 16.0;
-    if (lane < 16) f[lane] = (float)v;
 }
 
 // the smallest row length at least k times the mean (as FP64 compares them)
@@ -212,8 +216,15 @@ int run_features(const int32_t *row_ptr, int32_t m, int32_t n, int32_t nnz, floa
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     const double mean = m > 0 ? (double)nnz / (double)m : 0.0;
-    feature_kernel<<<(unsigned)blocks, kFeatThreads, 0, s>>>(row_ptr, m, nnz, at_least(2.0, mean),
-                                                            at_least(32.0, mean), cnt, out);
+    const double md = m > 0 ? (double)m : 1.0;
+    HostFeatures h;
+    h.mean = (double)nnz / md;
+    h.f0 = (float)(std::log2(md + 1.0) / 24.0);
+    h.f1 = (float)(std::log2((double)nnz + 1.0) / 32.0);
+    h.f2 = (float)(std::log2(h.mean + 1.0) / 8.0);
+    h.f13 = (float)(std::log2(480.0 / (h.mean + 1e-9) + 1.0) / 16.0);  // rows per 480-entry tile
+    feature_kernel<<<(unsigned)blocks, kFeatThreads, 0, s>>>(
+        row_ptr, m, nnz, at_least(2.0, mean), at_least(32.0, mean), h, cnt, out);
     e = cudaGetLastError();
     if (e != cudaSuccess) return record_cuda_error(e);
     return SSSPMV_OK;
@@ -340,7 +351,7 @@ __global__ void argmin_kernel(const float *__restrict__ out, int B, int K, int32
 // mlp_reduce_kernel adds the blocks' shares in order.  One layer per launch
 // and one thread per weight over the whole batch took 960 us for a training
 // step on 2,000 samples, nearly all of it the weight gradients' serial sums;
-// this takes 20.
+// this takes 14.
 
 constexpr int kMlpH = 64, kMlpMaxF = 32, kMlpMaxK = 32, kMlpTile = 16;
 constexpr int kMlpLd = kMlpH + 4;  // rows of 64 a bank group apart, 16-byte aligned
@@ -371,6 +382,7 @@ struct MlpArgs {
 __device__ __forceinline__ void mlp_dot4(float (&acc)[4], const float (*W)[kMlpLd], int o,
                                          const float *in, int ld, int n)
 {
+#pragma unroll 4
     for (int i = 0; i < n; i += 4) {
         const float w0 = W[i][o], w1 = W[i + 1][o], w2 = W[i + 2][o], w3 = W[i + 3][o];
 #pragma unroll
@@ -396,10 +408,14 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_kernel(const MlpArgs a)
     grid_dep_wait();  // the parameters may come from the kernel before
     grid_dep_trigger();
     for (int k = t; k < H * F; k += kMlpThreads) s.W1t[k % F][k / F] = __ldg(W1 + k);
-    for (int k = t; k < H * H; k += kMlpThreads) {
-        const float w = __ldg(W2 + k);
-        s.W2[k / H][k % H] = w;
-        s.W2t[k % H][k / H] = w;
+    float w2[H * H / kMlpThreads];  // all on their way at once
+#pragma unroll
+    for (int q = 0; q < H * H / kMlpThreads; ++q) w2[q] = __ldg(W2 + t + q * kMlpThreads);
+#pragma unroll
+    for (int q = 0; q < H * H / kMlpThreads; ++q) {
+        const int k = t + q * kMlpThreads;
+        s.W2[k / H][k % H] = w2[q];
+        s.W2t[k % H][k / H] = w2[q];
     }
     for (int k = t; k < K * H; k += kMlpThreads) s.W3[k / H][k % H] = __ldg(W3 + k);
     if (t < H) {
@@ -435,7 +451,15 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_kernel(const MlpArgs a)
         for (int k = t; k < kMlpTile * K; k += kMlpThreads) {
             const int b = k / K, c = k % K;
             float v = s.b3[c];
-            for (int i = 0; i < H; ++i) v = fmaf(s.W3[c][i], s.a2[b][i], v);
+#pragma unroll
+            for (int i = 0; i < H; i += 4) {
+                const float4 w = *reinterpret_cast<const float4 *>(&s.W3[c][i]);
+                const float4 h = *reinterpret_cast<const float4 *>(&s.a2[b][i]);
+                v = fmaf(w.x, h.x, v);
+                v = fmaf(w.y, h.y, v);
+                v = fmaf(w.z, h.z, v);
+                v = fmaf(w.w, h.w, v);
+            }
             s.o3[b][c] = v;
             float g = 0.0f;
             if (b0 + b < a.B) {
