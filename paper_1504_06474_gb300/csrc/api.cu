@@ -144,7 +144,7 @@ static int make_layout(int32_t m, int32_t nnz, int32_t val_bytes, const ssspmv_o
     carve(l);
     // the lists of the row blocks outgrow the records of BF16's longer tiles
     if (val_bytes == 2 && automatic(o)) {
-        const RowShape s = row_shape(m, nnz);
+        const RowShape s = row_shape(m, nnz, val_bytes);
         const size_t need = l.off_tile_offset + row_lists(nnz, s.cap, s.piece).bytes;
         if (l.total < need) l.total = align256(need);
     }
@@ -155,9 +155,10 @@ static int make_layout(int32_t m, int32_t nnz, int32_t val_bytes, const ssspmv_o
 // shape, bunch size, block size or variant: the segmented sum over tiles
 // remains for those who do.  Their lists live in the sections the tiles'
 // records take otherwise; a layout too small for them keeps the tiles.
-static bool takes_rows(int32_t m, int32_t nnz, const ssspmv_opts *o, const Layout &l)
+static bool takes_rows(int32_t val_bytes, int32_t m, int32_t nnz, const ssspmv_opts *o,
+                       const Layout &l)
 {
-    return automatic(o) && row_lists_fit(nnz, row_shape(m, nnz), l);
+    return automatic(o) && row_lists_fit(nnz, row_shape(m, nnz, val_bytes), l);
 }
 
 static bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
@@ -321,7 +322,7 @@ static int run_call(int32_t val_bytes, int32_t m, int32_t n, int32_t nnz,
         c.beta = beta;
         c.axpby = 1;
     }
-    if (!tiles_only && takes_rows(m, nnz, opts, l)) {
+    if (!tiles_only && takes_rows(val_bytes, m, nnz, opts, l)) {
         c.rows = 1;
         if (header != kHeaderClear) {
             cudaError_t e = cudaMemsetAsync(c.ws + l.off_err, 0, kHeaderBytes, c.stream);
@@ -601,7 +602,7 @@ int ssspmv_plan_create(int32_t m, int32_t n, int32_t nnz, const int32_t *row_ptr
     p->lay = l;
     p->exact = (opts && opts->variant == SSSPMV_VARIANT_EXACT) ? 1 : 0;
     p->block_warps = opts ? opts->block_warps : 0;
-    p->rows = takes_rows(m, nnz, opts, l) ? 1 : 0;
+    p->rows = takes_rows(val_bytes, m, nnz, opts, l) ? 1 : 0;
     if (workspace && (ws_bytes < l.total || ((uintptr_t)workspace & 255u))) {
         delete p;
         return SSSPMV_EWORKSPACE;
@@ -801,7 +802,7 @@ int ssspmv_csr_f64_debug(int32_t m, int32_t n, int32_t nnz, const int32_t *row_p
     rc = ssspmv_device_status(workspace, ws_bytes, stream, 0, &bits);
     if (rc) return rc;
     if (bits) return SSSPMV_EDEVICE;
-    if (!takes_rows(m, nnz, opts, l)) return SSSPMV_OK;
+    if (!takes_rows(8, m, nnz, opts, l)) return SSSPMV_OK;
     // ssspmv_csr_f64 with these options goes by row blocks: y is its y
     rc = run_call(8, m, n, nnz, row_ptr, col_idx, val, x, y, opts, workspace, ws_bytes, stream,
                   nullptr, nullptr, nullptr);

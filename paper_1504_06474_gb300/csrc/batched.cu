@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(kPrepThreads)
             continue;
         }
         nt += ((int64_t)d.nnz + L - 1) / L;
-        nu += row_units(d.m, row_shape(d.m, d.nnz)).nunits;
+        nu += row_units(d.m, row_shape(d.m, d.nnz, 4)).nunits;
     }
     if (bad) atomicOr(head + kWordErr, SSSPMV_DEV_BATCH);
     int64_t tot_t = 0, tot_u = 0;
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kPrepThreads)
         DescView d = desc[i];
         if (!valid_desc(d) || !fits)
             d = DescView{0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, nullptr};
-        const RowShape s = row_shape(d.m, d.nnz);
+        const RowShape s = row_shape(d.m, d.nnz, 4);
         const RowUnits u = row_units(d.m, s);
         RowMat r;
         r.val = d.val;

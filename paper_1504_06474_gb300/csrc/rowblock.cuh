@@ -36,8 +36,8 @@
 namespace ssspmv {
 
 // ---------------------------------------------------------------------------
-// shape of the row blocks, from m and nnz alone (so a batch and a single call
-// agree on it, and with it on every sum's order)
+// shape of the row blocks, from m, nnz and the value type alone (so a batch and
+// a single call agree on it, and with it on every sum's order)
 
 struct RowShape {
     int32_t gs;     // log2 of the lanes per row
@@ -52,21 +52,27 @@ constexpr int32_t kStageMax = 888;
 
 constexpr int32_t kMinCap = 640, kMinPiece = 10;
 
-__host__ __device__ inline RowShape row_shape(int32_t m, int32_t nnz)
+__host__ __device__ inline RowShape row_shape(int32_t m, int32_t nnz, int32_t val_bytes)
 {
     RowShape s;
     const int64_t mm = m > 0 ? m : 1;
     // one lane per row up to 27 entries on average (a 27-point stencil's 864
     // entries per group just fit), then 14 to 27 entries per lane; and more
-    // lanes where the groups would be too few to keep every warp busy
+    // lanes where the groups would be too few to keep every warp busy (uniform
+    // rows of 0..40 entries, 120,007 of them, FP64: 24 us with two lanes, 27
+    // with one).  In FP32 far fewer groups are left whole, because the matrices
+    // of a batch share the GPU: 96 mixed ones take 297 to 317 us below 1,536
+    // groups, 397 with FP64's rule, and single small ones are as fast
+    const int64_t few = val_bytes == 8 ? 6144 : 384;
     s.gs = 0;
     while (s.gs < 5 && (int64_t)nnz > ((int64_t)27 << s.gs) * mm) ++s.gs;
-    while (s.gs < 5 && (mm >> (5 - s.gs)) < 6144 && (int64_t)nnz > ((int64_t)8 << s.gs) * mm)
+    while (s.gs < 5 && (mm >> (5 - s.gs)) < few && (int64_t)nnz > ((int64_t)8 << s.gs) * mm)
         ++s.gs;
     // four groups at a time, where that leaves enough units for every warp
-    s.us = (mm >> (7 - s.gs)) >= 6144 ? 2 : 0;
-    // room for groups well above the mean, and for several short ones
+    // (half as many where several groups share a copy)
     const int64_t group = ((int64_t)nnz << (5 - s.gs)) / mm;  // its mean entries
+    s.us = (mm >> (7 - s.gs)) >= (group <= 320 ? 3072 : 6144) ? 2 : 0;
+    // room for groups well above the mean, and for several short ones
     int64_t cap = (group + group / 2) & ~(int64_t)7;
     if (cap < kMinCap) cap = kMinCap;
     if (cap > kStageMax) cap = kStageMax;
@@ -197,6 +203,7 @@ __device__ __forceinline__ typename P::acc_t lane_dot(const typename P::val_t *v
 }
 
 constexpr int kUnitRowsMax = 128;
+constexpr int kBatchRowWarps = 20;  // a batch's kernel needs 96 registers
 
 struct alignas(16) RowScratch {
     uint64_t bar;
@@ -377,7 +384,7 @@ __device__ __forceinline__ int32_t inside(int32_t p, int32_t b, int32_t e)
 }
 
 template <class P, bool MULTI, bool BATCHED = false>
-__global__ void __launch_bounds__(P::kRowWarps * 32, 1)
+__global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32, 1)
     rowblock_kernel(const RowArgs a, int32_t stage_bytes, int32_t col_off)
 {
     using V = typename P::val_t;
@@ -933,7 +940,8 @@ int launch_rowblock(const Call &c, const RowArgs &a)
     // than grids.
     const int32_t budget = ((int64_t)a.nnz > 4 * (int64_t)a.m ? 194 : 162) * 1024;
     const StageShape s = stage_shape<P>(a.shape.cap, budget);
-    int32_t warps = s.warps < P::kRowWarps ? s.warps : P::kRowWarps;
+    constexpr int32_t most = BATCHED ? kBatchRowWarps : P::kRowWarps;
+    int32_t warps = s.warps < most ? s.warps : most;
     const int sms = device_sm_count();
     const unsigned grid = (unsigned)(a.nunits < sms ? a.nunits : sms);
     const int32_t need = (int32_t)((a.nunits + (int64_t)grid - 1) / grid);
@@ -985,7 +993,7 @@ int run_rowblock(const Call &c)
     if (c.ev && (e = cudaEventRecord(c.ev[1], c.stream)) != cudaSuccess)
         return record_cuda_error(e);
     RowArgs a;
-    a.shape = row_shape(c.m, c.nnz);
+    a.shape = row_shape(c.m, c.nnz, (int32_t)sizeof(typename P::val_t));
     const RowLists rl = row_lists(c.nnz, a.shape.cap, a.shape.piece);
     unsigned char *lists = c.ws + c.lay.off_tile_offset;
     a.row_ptr = c.row_ptr;
