@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kPrepThreads)
                            int64_t cap_tiles, RowMat *__restrict__ mats, uint32_t *head)
 {
     __shared__ int64_t warp_sums[32];
-    if (threadIdx.x < 8) head[threadIdx.x] = 0u;
+    if (threadIdx.x < kHeaderBytes / 4) head[threadIdx.x] = 0u;
     __syncthreads();
     const int32_t per = (count + kPrepThreads - 1) / kPrepThreads;
     const int32_t i0 = threadIdx.x * per;

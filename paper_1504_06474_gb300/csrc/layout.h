@@ -34,12 +34,13 @@ inline int32_t auto_bunch_tiles(int64_t ntiles)
 //                                  empty rows, cleared by kernel (c)
 //   [4,5] lengths of the lists of rows rowblock_kernel leaves to
 //         rowtail_kernel, [6] rowtail_kernel's ticket, [7] its finished
-//         blocks: zero between calls (rowtail_kernel clears them)
+//         blocks, [8] rowblock_kernel's ticket: zero between calls
+//         (rowtail_kernel clears them)
 // (a plan execution, which skips kernel (a), clears words 0..2 and keeps the
 // plan's flag)
 constexpr int kWordErr = 0, kWordTicket = 1, kWordDirty = 2, kWordSpread = 3;
-constexpr int kWordLists = 4, kWordTailTicket = 6, kWordTailDone = 7;
-constexpr size_t kHeaderBytes = 32;
+constexpr int kWordLists = 4, kWordTailTicket = 6, kWordTailDone = 7, kWordUnitTicket = 8;
+constexpr size_t kHeaderBytes = 64;
 
 struct Layout {
     int32_t W = 0, L = 0, S = 0;
@@ -104,7 +105,7 @@ inline void batch_layout(int32_t count, int64_t total_nnz, int32_t W, int32_t S,
     l.cap_bunches = (l.cap_tiles + S - 1) / S + count;
     size_t o = 0;
     l.off_err = o;  // err word, ticket, totals {tiles, bunches}, dirty-tile count
-    o = align256(o + 32);
+    o = align256(o + kHeaderBytes);
     l.off_mats = o;
     o = align256(o + kBatchMatBytes * (size_t)(count > 0 ? count : 1));
     l.off_toff = o;

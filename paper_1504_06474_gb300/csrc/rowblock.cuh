@@ -202,6 +202,7 @@ __device__ __forceinline__ typename P::acc_t lane_dot(const typename P::val_t *v
     return acc;
 }
 
+constexpr int kTurnUnits = 8192;  // fewer units are all taken by turns
 constexpr int kUnitRowsMax = 128;
 constexpr int kBatchRowWarps = 20;  // a batch's kernel needs 96 registers
 
@@ -429,10 +430,20 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
         piece = p >> 16;
     };
     const int32_t nunits = BATCHED ? __ldg(a.total_units) : a.nunits;
+    // The first quarter of the units by turns (block b takes every gridDim.x-th
+    // from the b-th on, its warps by a ticket in shared memory), the others by
+    // a ticket of the whole grid: the blocks' shares of a power-law matrix
+    // differ by a quarter of their time.  All of them by turns: R-MAT scale 22
+    // 145 us, scale 20 FP32 53; half 123 and 51; a quarter 118 and 47; none
+    // 118 and 49.  Small matrices would only wait for the ticket (120,007 rows
+    // of 0..40 entries: 23 us, 24 with it), and a batch's even each other out
+    // (342 us, 355 with half of them).
+    const bool turns = BATCHED || nunits < kTurnUnits;
+    const int64_t nstatic = turns ? INT64_MAX : nunits >> 2;
     const uint64_t pol_keep = policy_evict_last(), pol_stream = policy_evict_first();
 
-    // the block's next unit of rows [r0, r0 + nr): several groups at a time
-    // first, single ones towards the end; its row pointers are loaded into
+    // the next unit of rows [r0, r0 + nr): several groups at a time first,
+    // single ones towards the end; its row pointers are loaded into
     // registers, the lane's i-th being row_ptr[r0 + 32 i + lane]
     constexpr int NP = kUnitRowsMax / 32 + 1;
     struct Unit {
@@ -440,18 +451,22 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
         int32_t mat;
         int32_t rp[NP];
     };
-    int32_t at_mat = 0;  // the block's tickets only grow, and with them the matrix
+    int32_t at_mat = 0;  // a warp's tickets only grow, and with them the matrix
     auto next_unit = [&]() -> Unit {
-        int32_t t = 0;
-        if (lane == 0) t = atomicAdd(&s_ticket, 1);
+        uint32_t t = 0;
+        if (lane == 0) {
+            const int64_t turn = (int64_t)atomicAdd(&s_ticket, 1) * gridDim.x + blockIdx.x;
+            t = (uint32_t)(turn < nunits ? turn : nunits);
+            if (!BATCHED && turn >= nstatic)
+                t = (uint32_t)nstatic + atomicAdd(a.head + kWordUnitTicket, 1u);
+        }
         t = __shfl_sync(FULL, t, 0);
-        const int64_t u64 = (int64_t)t * gridDim.x + blockIdx.x;
         Unit q;
         q.r0 = -1;
         q.nr = 0;
         q.mat = 0;
-        if (u64 >= nunits) return q;
-        int32_t u = (int32_t)u64, um = m, ugs = gs, us = a.shape.us, nbig = a.nbig;
+        if (t >= (uint32_t)nunits) return q;
+        int32_t u = (int32_t)t, um = m, ugs = gs, us = a.shape.us, nbig = a.nbig;
         const int32_t *row_ptr = a.row_ptr;
         if constexpr (BATCHED) {
             while (at_mat + 1 < a.count && u >= __ldg(&a.mats[at_mat + 1].unit_base)) ++at_mat;
@@ -719,6 +734,7 @@ __global__ void __launch_bounds__(kTailThreads, BLOCKS) rowtail_kernel(const Row
     grid_dep_wait();
     uint32_t nr = *(volatile const uint32_t *)(a.head + kWordLists);
     uint32_t np = *(volatile const uint32_t *)(a.head + kWordLists + 1);
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.head[kWordUnitTicket] = 0u;  // (r1)'s
     if (nr + np == 0u) return;  // every row was staged
     // (an invalid row_ptr may have been refused more than the lists hold)
     nr = nr > (uint32_t)a.max_ranges ? 0u : nr;
@@ -737,23 +753,31 @@ __global__ void __launch_bounds__(kTailThreads, BLOCKS) rowtail_kernel(const Row
         return p < 0 ? 0 : (p > nnz ? nnz : p);
     };
     const uint32_t warps = gridDim.x * (kTailThreads / 32);
+    // The last ranges, half as many as there are warps, are shared by four
+    // warps each (eight if there are few), or most warps would wait for a few
+    // at the end (FP32, R-MAT scale 20: 56 us if none are shared, 52 so, 54 if
+    // as many as warps are, 62 if those by eight).
+    const uint32_t nsub = 8 * nr <= warps ? 8 : 4;
+    const uint32_t whole = nr > warps / 2 ? nr - warps / 2 : 0u;
+    // the first piece of work by the warp's place, the others by ticket
+    uint32_t w = blockIdx.x * (kTailThreads / 32) + (threadIdx.x >> 5);
+    const uint32_t total = np + whole + (nr - whole) * nsub;
+    // (drawing the next ticket early gave the last ones to busy warps: 56 -> 64 us)
     auto next = [&]() -> uint32_t {
         uint32_t t = 0;
         if (lane == 0) t = warps + atomicAdd(a.head + kWordTailTicket, 1u);
         return __shfl_sync(FULL, t, 0);
     };
-    // few ranges: several warps share one (a power of two, up to eight)
-    uint32_t nsub = 1;
-    while (nsub < 8 && 2 * nsub * nr <= warps) nsub *= 2;
-    // the first piece of work by the warp's place, the others by ticket
-    uint32_t w = blockIdx.x * (kTailThreads / 32) + (threadIdx.x >> 5);
-    for (; w < nr * nsub + np; w = next()) {
+    for (; w < total; w = next()) {
         // the entries [s, e) of the lane's row, row0 + lane; a piece of a very
         // long row: lane 0's
         const bool piece = w < np;
-        const int2 it = piece ? a.pieces[w] : a.ranges[(w - np) / nsub];
+        const bool shared = w >= np + whole;
+        const uint32_t ri = shared ? whole + (w - np - whole) / nsub : w - np;
+        const uint32_t sub = shared ? (w - np - whole) & (nsub - 1) : 0u;
+        const int2 it = piece ? a.pieces[w] : a.ranges[ri];
         if constexpr (BATCHED) {
-            const RowMat *mm = a.mats + (piece ? a.piece_mat[w] : a.range_mat[(w - np) / nsub]);
+            const RowMat *mm = a.mats + (piece ? a.piece_mat[w] : a.range_mat[ri]);
             val = static_cast<const V *>(ldg_ptr(&mm->val));
             x = static_cast<const X *>(ldg_ptr(&mm->x));
             y = static_cast<Y *>(ldg_ptr(const_cast<void *const *>(&mm->y)));
@@ -763,7 +787,6 @@ __global__ void __launch_bounds__(kTailThreads, BLOCKS) rowtail_kernel(const Row
             nnz = __ldg(&mm->nnz);
             pl = __ldg(&mm->packed) >> 16;
         }
-        const uint32_t sub = piece ? 0u : (w - np) & (nsub - 1);
         const bool in = piece ? lane == 0 : lane < it.y && it.x + lane < m;
         int32_t s = in ? rp(it.x + lane) : 0, e = in ? rp(it.x + lane + 1) : 0;
         const int32_t row_len = e - s;
@@ -803,7 +826,7 @@ __global__ void __launch_bounds__(kTailThreads, BLOCKS) rowtail_kernel(const Row
         // the longer rows, every nsub-th from the sub-th on, 32 * UN entries at a
         // time: the values and columns of a block of entries, be it the row's
         // or the next row's, are loaded while the block before it gathers
-        if (nsub > 1) {
+        if (shared) {
             unsigned mine = 0;
             for (uint32_t k = 0; todo; ++k, todo &= todo - 1)
                 if ((k & (nsub - 1)) == sub) mine |= todo & -todo;

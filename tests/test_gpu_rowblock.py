@@ -110,6 +110,20 @@ def test_f64_rounding(dev, kind):
     assert np.all(np.abs(y.cpu().numpy() - yref) <= 1e-13 * s)
 
 
+@pytest.mark.parametrize("m", [8191, 8192, 8193, 8400])
+def test_units_by_turns_and_by_ticket(dev, m):
+    """One row per unit, on both sides of where a grid-wide ticket hands them
+    out, several calls in one workspace (the ticket starts from zero again)."""
+    from paper_1504_06474_gb300 import ssspmv as C
+    rp, col, val, x = _matrix("const440", m, 997, seed=m)
+    nnz, want = int(rp[-1]), oracle.spmv(rp, col, val, x)
+    rpd, cd, vd, xd = _device(dev, (rp, col, val, x))
+    for _ in range(3):
+        y = torch.full((m,), -1.0, dtype=torch.float64, device=dev)
+        C.check(C.ssspmv_csr_f64(m, 997, nnz, rpd, cd, vd, xd, y), "csr")
+        np.testing.assert_array_equal(y.cpu().numpy(), want)
+
+
 @pytest.mark.parametrize("prec", ["f32", "bf16"])
 @pytest.mark.parametrize("kind", KINDS)
 def test_reduced_precision_equals_the_row_loop(dev, kind, prec):
