@@ -298,12 +298,17 @@ int run_batched_shape(int32_t count, const void *desc, const BatchLayout &l, uns
 
 // Set-up of a batch by row blocks (one block): checks the descriptors as above,
 // numbers the batch's units of rows and writes the records.  The capacity is
-// counted in tiles too, so the two ways accept the same batches.
+// counted in tiles too, so the two ways accept the same batches.  Bound by its
+// chain of loads and scans; launched like the others of the chain, so that the
+// launches before and after it overlap (8 matrices of 1,000 to 20,000 rows:
+// 28.8 -> 27.1 us a call).
 __global__ void __launch_bounds__(kPrepThreads)
     batch_rows_prep_kernel(const DescView *__restrict__ desc, int32_t count, int32_t L,
                            int64_t cap_tiles, RowMat *__restrict__ mats, uint32_t *head)
 {
     __shared__ int64_t warp_sums[32];
+    grid_dep_wait();
+    grid_dep_trigger();  // (r1) waits for this kernel with its blocks in place
     if (threadIdx.x < kHeaderBytes / 4) head[threadIdx.x] = 0u;
     __syncthreads();
     const int32_t per = (count + kPrepThreads - 1) / kPrepThreads;
@@ -374,9 +379,10 @@ static int run_batched_rows(int32_t count, const void *desc, const BatchLayout &
     a.range_mat = reinterpret_cast<int32_t *>(ws + l.off_rmat);
     a.piece_mat = reinterpret_cast<int32_t *>(ws + l.off_pmat);
     if (ev && (e = cudaEventRecord(ev[0], stream)) != cudaSuccess) return record_cuda_error(e);
-    batch_rows_prep_kernel<<<1, kPrepThreads, 0, stream>>>(
-        static_cast<const DescView *>(desc), count, l.L, l.cap_tiles,
-        reinterpret_cast<RowMat *>(ws + l.off_rmats), a.head);
+    e = launch_dependent(batch_rows_prep_kernel, 1, kPrepThreads, 0, stream,
+                         static_cast<const DescView *>(desc), count, l.L, l.cap_tiles,
+                         reinterpret_cast<RowMat *>(ws + l.off_rmats), a.head);
+    if (e != cudaSuccess) return record_cuda_error(e);
     if (ev && (e = cudaEventRecord(ev[1], stream)) != cudaSuccess) return record_cuda_error(e);
     Call c;
     c.stream = stream;
