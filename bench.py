@@ -9,9 +9,9 @@ and the plain FP64 call beside it; --workload batch<count> times the batched
 FP32 call over a seeded mixed batch as one CUDA-graph replay, beside the same
 matrices as separate FP32 calls and separate plain FP64 calls.
 
-A step is one full y = A x through ssspmv_csr_f64 (kernels (a) partition,
-(b) segmented sum, (c) calibration) on the synthetic 27-point stencil over a
-160^3 grid in FP64 (m = 4,096,000, nnz = 109,215,352), inputs resident in
+A step is one full y = A x through ssspmv_csr_f64 (by blocks of rows; with a
+tile shape or a variant, kernels (a) partition, (b) segmented sum and (c)
+calibration) on the synthetic 27-point stencil over a 160^3 grid in FP64 (m = 4,096,000, nnz = 109,215,352), inputs resident in
 HBM.  L2 is flushed (a 512 MB write, then a read) between timed steps, outside the timed
 events.  value = algorithmic bytes / time, bytes = nnz*(8+4) + (m+1)*4 +
 m*8 + n*8 (x read once), in GB/s.  Under torchrun each rank runs an
@@ -60,9 +60,41 @@ def peaks():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-# the sources that define kernel (b) and its launch (device code, tile shape,
-# workspace carve-up, block shape); host-only files do not change its traffic
-KERNEL_B_SOURCES = ("layout.h", "launch.cuh", "ptx.cuh", "segsum.cuh", "spmv_f64.cu")
+# the sources that define the product's kernels and their launches (device code,
+# tile and row-block shapes, workspace carve-up); host-only files do not change
+# their traffic
+KERNEL_B_SOURCES = ("layout.h", "launch.cuh", "ptx.cuh", "rowblock.cuh", "segsum.cuh",
+                    "spmv_f64.cu")
+
+
+def product_path(opts_kw: dict) -> dict:
+    """What a product with these options launches: the kernel that carries it,
+    the launches of one call, and the names of the timer's three stages.  With
+    everything automatic that is the two kernels of the row blocks (a batch's
+    set-up kernel before them), the second of which works off the rows the first
+    one leaves; with a tile shape or a variant, the segmented sum's kernels."""
+    if not any(opts_kw.get(k) for k in ("W", "S", "variant", "block_warps")):
+        return {"kernel": "rowblock_kernel", "launches": 2,
+                "stages": ("prepare", "rowblock", "rowtail")}
+    if opts_kw.get("variant") == 3:
+        return {"kernel": "csr_rows_kernel", "launches": 1,
+                "stages": ("partition", "segsum", "calibrate")}
+    return {"kernel": "segsum_kernel", "launches": 3,
+            "stages": ("partition", "segsum", "calibrate")}
+
+
+def stage_ms(path: dict, times) -> dict:
+    """Mean milliseconds of the timer's stages, and of the whole call."""
+    k = len(times)
+    d = {name: round(sum(t[i] for t in times) / k, 5) for i, name in enumerate(path["stages"])}
+    d["steps"] = k
+    d["whole"] = round(sum(t[3] for t in times) / k, 5)
+    return d
+
+
+def product_ms(path: dict, stages: dict) -> float:
+    """The part of the stages that streams the matrix."""
+    return sum(stages[n] for n in path["stages"] if n in ("rowblock", "rowtail", "segsum"))
 
 
 def source_digest() -> str:
@@ -306,7 +338,7 @@ def run_ours(args):
     clocks = sampler.stop()
 
     # stage breakdown: the library's own events at the kernel boundaries, in a
-    # run of its own (events between the kernels keep kernels (b) and (c)
+    # run of its own (events between the kernels keep the later kernels
     # from starting early, so these steps are a little longer)
     Ks = min(K, 200)
     timer = C.ssspmv_timer_create(Ks)
@@ -318,9 +350,9 @@ def run_ours(args):
     times = C.ssspmv_timer_read(timer, Ks)
     C.ssspmv_timer_destroy(timer)
     assert len(times) == Ks
-    part = [t[0] for t in times]                                             # ms
-    seg = [t[1] for t in times]
-    cal = [t[2] for t in times]
+    path = product_path({"W": args.tile_w, "S": args.tile_s, "variant": args.variant,
+                         "block_warps": args.block_warps})
+    stages = stage_ms(path, times)
     t_total = sum(per_step) / 1e3                                            # s
     if selected is not None:
         # the default configuration on the same matrix, timed the same way
@@ -338,7 +370,7 @@ def run_ours(args):
         selected["speedup_vs_default"] = round(d_ms / (t_total / K * 1e3), 4)
         del ws_d
         step(plain)  # y from the selected configuration again
-    # plan reuse (partition once; kernels (b) and (c) per product, the
+    # plan reuse (what depends on row_ptr alone computed once, the
     # iterative-solver form), timed the same way beside the one-shot call,
     # with y checked against it
     plan_ms = None
@@ -396,12 +428,10 @@ def run_ours(args):
         raise RuntimeError("device status bits %#x" % status)
 
     hbm, peak_kind = peaks()
-    seg_ms = sum(seg) / Ks
-    achieved = nbytes / (seg_ms / 1e3) / 1e9
-    # the ncu record holds for the default configuration it was captured with
-    default_cfg = (not args.select and args.tile_w in (0, 15) and args.variant == 0
-                   and args.block_warps == 0 and args.tile_s in (0, 4))
-    traffic = ncu_traffic("segsum_kernel", args.workload) if default_cfg else None
+    achieved = nbytes / (product_ms(path, stages) / 1e3) / 1e9
+    # the ncu record holds for the configuration it was captured with, all automatic
+    default_cfg = path["kernel"] == "rowblock_kernel"
+    traffic = ncu_traffic(path["kernel"], args.workload) if default_cfg else None
     line = None
     if rank == 0:
         cpu = None
@@ -426,26 +456,22 @@ def run_ours(args):
                        "gflops": round(2.0 * A.nnz * K * world / t_total / 1e9, 3),
                        "l2": ("not flushed (hot: inputs stay in L2 between steps)" if args.hot else
                               "flushed between steps (512 MB write then read, outside the timed events)"),
-                       "stage_ms": {"partition": round(sum(part) / Ks, 5),
-                                    "segsum": round(seg_ms, 5),
-                                    "calibrate": round(sum(cal) / Ks, 5),
-                                    "steps": Ks,
-                                    "whole": round(sum(t[3] for t in times) / Ks, 5)},
+                       "stage_ms": stages,
                        "plan_reuse": None if plan_ms is None else {
                            "ms_per_step": round(plan_ms, 5),
                            "value": round(nbytes / (plan_ms / 1e3) / 1e9, 3), "unit": "GB/s",
                            "hbm_frac": round(nbytes / (plan_ms / 1e3) / 1e9 / hbm, 4),
-                           "steps": Ks, "what": "ssspmv_plan_execute: kernels (b) and (c) on "
-                                               "a partition computed once"},
+                           "steps": Ks, "what": "ssspmv_plan_execute: the product's kernels "
+                                               "with what depends on row_ptr computed once"},
                        "wall_s_timed_loop": round(t_wall, 3)},
             "roofline": {"bound": "hbm",
-                         "kernel": "csr_rows_kernel" if rows_variant else "segsum_kernel",
+                         "kernel": path["kernel"],
                          "achieved": round(achieved, 2), "peak": hbm, "unit": "GB/s",
                          "frac": round(achieved / hbm, 4), "peak_kind": peak_kind,
                          "traffic": traffic},
             "clocks": clocks,
             "e2e": e2e,
-            "gpu_launches": (1 if rows_variant else 3) * K,
+            "gpu_launches": path["launches"] * K,
             "cpu_baseline": cpu,
         }
         if world == 1 and args.configs and args.workload == "stencil160" and not args.select:
@@ -601,18 +627,15 @@ def _time_whole(step, K, flush_l2, stream, gpu, warmup=3):
 
 
 def _stages(single, opts_kw, ws, K, flush_l2, stream):
-    """Kernel (a), (b), (c) and whole times (ms) from the library's events
-    at the kernel boundaries, in a run of their own."""
+    """The stages' and the whole times (ms) from the library's events at the
+    kernel boundaries, in a run of their own."""
     from paper_1504_06474_gb300 import ssspmv as C
     timer = C.ssspmv_timer_create(K)
     ot = C.make_opts(timer=timer, **opts_kw)
     _timed_loop(lambda: single.call(ot, ws, stream), flush_l2, K, stream)
     t = C.ssspmv_timer_read(timer, K)
     C.ssspmv_timer_destroy(timer)
-    return {"partition": round(sum(v[0] for v in t) / K, 5),
-            "segsum": round(sum(v[1] for v in t) / K, 5),
-            "calibrate": round(sum(v[2] for v in t) / K, 5), "steps": K,
-            "whole": round(sum(v[3] for v in t) / K, 5)}
+    return stage_ms(product_path(opts_kw), t)
 
 
 def _errors(single, x64):
@@ -653,6 +676,8 @@ def measure_single(A, x, dev, precision, opts_kw, K, workload, cpu_seconds=0.0, 
     whole, med, clocks = _time_whole(lambda: single.call(opts, ws, stream), K, flush_l2, stream,
                                      gpu)
     st = _stages(single, opts_kw, ws, min(K, 200), flush_l2, stream)
+    path = product_path(opts_kw)
+    st_ms = product_ms(path, st)
     nbytes = single.nbytes
     value = nbytes / (whole / 1e3) / 1e9
     hbm, peak_kind = peaks()
@@ -669,11 +694,11 @@ def measure_single(A, x, dev, precision, opts_kw, K, workload, cpu_seconds=0.0, 
                    "ms_per_step_median": round(med, 5), "stage_ms": st,
                    "l2": ("not flushed (hot: inputs stay in L2 between steps)" if hot else
                           "flushed between steps (512 MB write then read, outside the timed events)")},
-        "roofline": {"bound": "hbm", "kernel": "segsum_kernel",
-                     "achieved": round(nbytes / (st["segsum"] / 1e3) / 1e9, 2), "peak": hbm,
-                     "unit": "GB/s", "frac": round(nbytes / (st["segsum"] / 1e3) / 1e9 / hbm, 4),
+        "roofline": {"bound": "hbm", "kernel": path["kernel"],
+                     "achieved": round(nbytes / (st_ms / 1e3) / 1e9, 2), "peak": hbm,
+                     "unit": "GB/s", "frac": round(nbytes / (st_ms / 1e3) / 1e9 / hbm, 4),
                      "peak_kind": peak_kind, "traffic": None},
-        "clocks": clocks, "gpu_launches": 3 * K,
+        "clocks": clocks, "gpu_launches": path["launches"] * K,
     }
     if precision != "f64":
         line["config"]["accumulation"] = "compensated FP32 pairs (TwoProduct + TwoSum)"
@@ -925,9 +950,12 @@ def measure_batch(args, dev):
         _timed_loop(lambda: batched(ot), flush_l2, kst, s)
     st = C.ssspmv_timer_read(timer, kst)
     C.ssspmv_timer_destroy(timer)
-    seg = sum(v[1] for v in st) / kst
-    stage = {"setup_and_partition": round(sum(v[0] for v in st) / kst, 5), "segsum": round(seg, 5),
-             "calibrate": round(sum(v[2] for v in st) / kst, 5)}
+    path = product_path({"W": args.tile_w, "S": args.tile_s, "variant": args.variant,
+                         "block_warps": bwarps})
+    path["stages"] = ("setup",) + path["stages"][1:] if path["launches"] == 2 else (
+        "setup_and_partition",) + path["stages"][1:]
+    stage = stage_ms(path, st)
+    seg = product_ms(path, stage)
     # the same matrices as separate single calls: FP32, and the plain FP64 kernel
     big = max(C.ssspmv_workspace_bytes(A.m, A.nnz, 8, None) for A, _ in mats)
     ws1 = torch.empty(big, dtype=torch.uint8, device=dev)
@@ -997,19 +1025,23 @@ def measure_batch(args, dev):
                    "W": C.ssspmv_plan_shape(1, 1, 4, opts)["W"],
                    "variant": ["default", "speculative", "exact", "rows"][args.variant],
                    "autotuned": tuned,
-                   "launch": "one CUDA graph replay: set-up, partition, one persistent "
-                             "segmented-sum launch over every bunch of every matrix, calibration",
+                   "launch": "one CUDA graph replay: set-up, then " + (
+                       "the row blocks of every matrix in one launch, and the rows it leaves"
+                       if path["launches"] == 2 else
+                       "partition, one persistent segmented-sum launch over every bunch of "
+                       "every matrix, calibration"),
                    "stage_ms": stage, "separate_f32_calls_ms": round(ms_sep, 4),
                    "speedup_vs_separate_f32_calls": round(ms_sep / ms, 3),
                    "separate_plain_f64_calls_ms": round(ms64, 4),
                    "speedup_vs_plain_f64": round(ms64 / ms, 3),
                    "generation_s": round(t_gen, 1),
                    "l2": "flushed between steps (512 MB write then read, outside the timed events)"},
-        "roofline": {"bound": "hbm", "kernel": "segsum_kernel (batched)",
+        "roofline": {"bound": "hbm", "kernel": path["kernel"] + " (batched)",
                      "achieved": round(nbytes / (seg / 1e3) / 1e9, 2), "peak": hbm,
                      "unit": "GB/s", "frac": round(nbytes / (seg / 1e3) / 1e9 / hbm, 4),
                      "peak_kind": peak_kind, "traffic": None},
-        "clocks": clocks, "e2e": e2e, "gpu_launches": 4 * K, "cpu_baseline": cpu,
+        "clocks": clocks, "e2e": e2e, "gpu_launches": (path["launches"] + 1) * K,
+        "cpu_baseline": cpu,
     }
     return line
 

@@ -42,7 +42,7 @@ F, H1, H2 = 16, 64, 64
 
 # (name, opts fields).  Class 0 is the fixed default: all library defaults.
 CLASSES = [
-    ("speculative W15 (default)", dict()),
+    ("row blocks (default)", dict()),
     ("speculative W21", dict(W=21, variant=C.VARIANT_SPECULATIVE)),
     ("speculative W27", dict(W=27, variant=C.VARIANT_SPECULATIVE)),
     ("speculative W31", dict(W=31, variant=C.VARIANT_SPECULATIVE)),
@@ -144,12 +144,12 @@ def autotune(Ad: DeviceMatrix, timer: Timer, reps: int = 3) -> np.ndarray:
 
 
 def tune_batched(count: int, desc, total_nnz: int, dev, reps: int = 3):
-    """The autotuner for a batch (ssspmv_csr_batched_f32): times every
-    compiled tile shape with speculative and exact stores on this batch and
-    returns (opts fields of the fastest, {name: ms})."""
+    """The autotuner for a batch (ssspmv_csr_batched_f32): times the row blocks
+    and every compiled tile shape with speculative and exact stores on this
+    batch and returns (opts fields of the fastest, {name: ms})."""
     import torch
     timer = Timer(dev)
-    cands = {}
+    cands = {"row blocks": dict(W=0, variant=C.VARIANT_DEFAULT)}
     for W in C.ssspmv_supported_w():
         for variant in (C.VARIANT_SPECULATIVE, C.VARIANT_EXACT):
             cands["W%d %s" % (W, "exact" if variant == C.VARIANT_EXACT else "speculative")] = \
