@@ -145,7 +145,8 @@ int ssspmv_plan_shape(int32_t m, int32_t nnz, int32_t val_bytes, const ssspmv_op
 
 /* Bytes of device workspace needed by a call with these arguments
  * (tile offsets, per-tile info, synchronizer records; the paper's
- * pre-allocated containers, Sec. 3.3).  Returns 0 on invalid arguments. */
+ * pre-allocated containers, Sec. 3.3; products by blocks of rows keep their
+ * lists of long rows in the same bytes).  Returns 0 on invalid arguments. */
 size_t ssspmv_workspace_bytes(int32_t m, int32_t nnz, int32_t val_bytes, const ssspmv_opts *opts);
 
 /* y = A x in FP64 (val, x, y double).  workspace: device buffer of at least
@@ -153,7 +154,8 @@ size_t ssspmv_workspace_bytes(int32_t m, int32_t nnz, int32_t val_bytes, const s
  * by another call in flight -- or NULL (ws_bytes ignored) for a buffer the
  * library owns, cached per (device, stream) and grown stream-ordered with
  * cudaMallocAsync on `stream` when a call needs more (see
- * ssspmv_cached_workspace).  Kernels: (a), (b), (c) above. */
+ * ssspmv_cached_workspace).  Kernels: by blocks of rows, or (a), (b), (c)
+ * above (see SSSPMV_VARIANT_DEFAULT). */
 int ssspmv_csr_f64(int32_t m, int32_t n, int32_t nnz,
                    const int32_t *row_ptr, const int32_t *col_idx, const double *val,
                    const double *x, double *y,
@@ -199,19 +201,22 @@ void ssspmv_release_workspaces(void);
 /* Partition reuse for iterative solvers (one sparsity pattern, many
  * products).  The paper has no plan -- its method needs no preprocessing
  * (Sec. 1), and the single calls above are what the headline numbers time --
- * but kernel (a) depends on row_ptr alone, so a plan runs it once:
+ * but kernel (a) depends on row_ptr alone, so a plan runs it once (a plan
+ * whose products go by blocks of rows has no kernel (a) to save: it saves the
+ * checks and the reset of the workspace):
  *   ssspmv_plan_create  checks the arguments, resolves the tile shape for the
  *     stored value type (val_bytes 8, 4 or 2; opts as for the single calls,
  *     opts->timer must be NULL), takes `workspace` (NULL: the plan allocates
- *     one with cudaMalloc and owns it) and launches kernel (a) on `stream`.
+ *     one with cudaMalloc and owns it) and launches kernel (a), or the reset
+ *     of the workspace's header, on `stream`.
  *     row_ptr stays the caller's: it must remain valid and unchanged while
- *     the plan lives (kernel (b) reads it on every execution).
- *   ssspmv_plan_execute  y = A x with the plan's partition: kernels (b) and
- *     (c) on `stream`, for col_idx/val/x/y of the plan's value type (double,
- *     float, or bf16 val with float x and y).  It allocates nothing; `timer`
+ *     the plan lives (every execution reads it).
+ *   ssspmv_plan_execute  y = A x on `stream` with the plan's partition
+ *     (kernels (b) and (c)) or by blocks of rows, for col_idx/val/x/y of the
+ *     plan's value type (double, float, or bf16 val with float x and y).  It allocates nothing; `timer`
  *     (nullable ssspmv_timer*) records it, its kernel (a) slot then timing the
- *     reset of the error word.  Executions of one plan share its workspace:
- *     order them on one stream.  Must run on the plan's device.
+ *     reset of the error word (by blocks of rows: nothing).  Executions of one
+ *     plan share its workspace: order them on one stream.  Must run on the plan's device.
  *   ssspmv_plan_workspace  the plan's workspace (for ssspmv_device_status).
  *   ssspmv_plan_destroy  frees what the plan owns (cudaFree: waits for the
  *     device). */

@@ -201,13 +201,15 @@ struct CachedWs {
     void *base;    // what cudaMallocAsync returned
     void *ptr;     // 256-byte aligned start
     size_t bytes;  // usable bytes from ptr
+    bool shown;    // the caller has the pointer: its header may hold anything
 };
 std::mutex g_ws_mutex;
 std::vector<CachedWs> g_ws;
 }  // namespace
 
-static int cached_workspace(size_t need, void *stream, void **ptr, size_t *bytes)
+static int cached_workspace(size_t need, void *stream, void **ptr, size_t *bytes, bool *shown)
 {
+    *shown = false;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return record_cuda_error(e);
@@ -219,6 +221,7 @@ static int cached_workspace(size_t need, void *stream, void **ptr, size_t *bytes
     if (slot && slot->bytes >= need) {
         *ptr = slot->ptr;
         *bytes = slot->bytes;
+        *shown = slot->shown;
         return SSSPMV_OK;
     }
     if (slot && slot->base) {
@@ -231,13 +234,14 @@ static int cached_workspace(size_t need, void *stream, void **ptr, size_t *bytes
     void *base = nullptr;
     if ((e = cudaMallocAsync(&base, want, s)) != cudaSuccess) return record_cuda_error(e);
     if (!slot) {
-        g_ws.push_back(CachedWs{dev, stream, nullptr, nullptr, 0});
+        g_ws.push_back(CachedWs{dev, stream, nullptr, nullptr, 0, false});
         slot = &g_ws.back();
     }
     const uintptr_t a = ((uintptr_t)base + 255u) & ~(uintptr_t)255u;
     slot->base = base;
     slot->ptr = reinterpret_cast<void *>(a);
     slot->bytes = want - (a - (uintptr_t)base);
+    slot->shown = false;
     // the error words at the front start cleared (kernel (b)'s schedule
     // flag is read before the first call's kernel (c) clears it)
     if ((e = cudaMemsetAsync(slot->ptr, 0, kHeaderBytes, s)) != cudaSuccess) return record_cuda_error(e);
@@ -267,9 +271,10 @@ static int run_call(int32_t val_bytes, int32_t m, int32_t n, int32_t nnz,
     if (out_layout) *out_layout = l;
     if (m == 0) return SSSPMV_OK;
     if (!ws) {
-        rc = cached_workspace(l.total, stream, &ws, &ws_bytes);
+        bool shown;
+        rc = cached_workspace(l.total, stream, &ws, &ws_bytes, &shown);
         if (rc) return rc;
-        header = kHeaderClear;  // between calls
+        if (!shown) header = kHeaderClear;  // between calls
     }
     if (ws_bytes < l.total || ((uintptr_t)ws & 255u)) return SSSPMV_EWORKSPACE;
     if (opts && opts->variant == SSSPMV_VARIANT_ROWS) {
@@ -704,7 +709,10 @@ int ssspmv_cached_workspace(void *stream, void **ptr, size_t *bytes)
     std::lock_guard<std::mutex> lock(g_ws_mutex);
     for (auto &w : g_ws)
         if (w.dev == dev && w.stream == stream && w.ptr) {
-            if (ptr) *ptr = w.ptr;
+            if (ptr) {
+                *ptr = w.ptr;
+                w.shown = true;
+            }
             if (bytes) *bytes = w.bytes;
             return SSSPMV_OK;
         }

@@ -21,12 +21,13 @@
 // row lengths are too uneven for that split their entries evenly over the
 // lanes instead (a segmented sum inside the group).
 //
-// Measured (us a call among others, FP64, before: the three kernels of
-// segsum.cuh): 27-point stencil 160^3 272 -> 245 (the FP64 pipe alone needs
-// 207), R-MAT scale 22 with a 10^6-entry row 405 -> 363, banded half-width 31
-// (300,001 rows, plan) 64 -> 53, uniform rows of 0..40 entries (120,007 rows,
-// axpby) 40 -> 23, rows of 1..8 entries and three of 500,000 92 -> 64,
-// uniform 4096 rows 17 -> 14.
+// Measured (us a call among others; before: the three kernels of segsum.cuh).
+// FP64: 27-point stencil 160^3 272 -> 241 (the FP64 pipe alone needs 207), R-MAT
+// scale 22 with a 10^6-entry row 404 -> 330, banded half-width 31 (300,001 rows,
+// plan) 64 -> 51, uniform rows of 0..40 entries (120,007 rows, axpby) 43 -> 23,
+// rows of 1..8 entries and three of 500,000 91 -> 65, uniform 4096 rows 15 -> 7.
+// FP32: stencil 101x97x103 62 -> 45, R-MAT scale 20 110 -> 91, 96 mixed matrices
+// 520 -> 337; BF16 values: stencil 120x125x131 110 -> 71.
 #pragma once
 #include <cstdint>
 
@@ -310,8 +311,9 @@ static __device__ __noinline__ void list_group(const RowArgs &a, int32_t mat, in
         got = atomicAdd(reinterpret_cast<unsigned long long *>(a.head + kWordLists),
                         ((unsigned long long)total << 32) | (unsigned)__popc(leads));
     got = __shfl_sync(FULL, got, 0);
-    const int32_t rbase = (int32_t)(got & 0xffffffffu), pbase = (int32_t)(got >> 32);
-    if (rbase + __popc(leads) > a.max_ranges || pbase + total > a.max_pieces) {
+    const uint32_t rbase = (uint32_t)got, pbase = (uint32_t)(got >> 32);
+    if ((uint64_t)rbase + __popc(leads) > (uint32_t)a.max_ranges ||
+        (uint64_t)pbase + (uint32_t)total > (uint32_t)a.max_pieces) {
         // more than any valid row_ptr can list
         if (lane == 0) atomicOr(a.head + kWordErr, SSSPMV_DEV_RANGE);
         return;
@@ -319,7 +321,7 @@ static __device__ __noinline__ void list_group(const RowArgs &a, int32_t mat, in
     if (lead) {
         const unsigned above = lane == 31 ? 0u : leads & ~((2u << lane) - 1u);
         const int next = above ? __ffs(above) - 1 : rows;
-        const int32_t at = rbase + __popc(leads & ((1u << lane) - 1u));
+        const uint32_t at = rbase + __popc(leads & ((1u << lane) - 1u));
         a.ranges[at] = make_int2(row0 + lane, next - lane);
         if (a.range_mat) a.range_mat[at] = mat;
     }
@@ -328,7 +330,7 @@ static __device__ __noinline__ void list_group(const RowArgs &a, int32_t mat, in
         const int src = __ffs(todo) - 1;
         todo &= todo - 1;
         const int32_t n = __shfl_sync(FULL, np, src);
-        const int32_t at = pbase + __shfl_sync(FULL, pincl, src) - n;
+        const uint32_t at = pbase + __shfl_sync(FULL, pincl, src) - n;
         if (lane == 0) a.arrived[at] = 0u;
         for (int32_t p = lane; p < n; p += 32) {
             a.pieces[at + p] = make_int2(row0 + src, p);
@@ -787,14 +789,17 @@ __global__ void __launch_bounds__(kTailThreads, BLOCKS) rowtail_kernel(const Row
             nnz = __ldg(&mm->nnz);
             pl = __ldg(&mm->packed) >> 16;
         }
-        const bool in = piece ? lane == 0 : lane < it.y && it.x + lane < m;
+        // (whatever the lists hold, nothing outside the arrays is touched)
+        const bool in = (piece ? lane == 0 : lane < it.y) &&
+                        (uint32_t)it.x + (uint32_t)lane < (uint32_t)m;
         int32_t s = in ? rp(it.x + lane) : 0, e = in ? rp(it.x + lane + 1) : 0;
         const int32_t row_len = e - s;
         unsigned todo;
         if (piece) {
-            s += it.y << pl;
+            const bool mine = (uint32_t)it.y <= w && it.y < (row_len + (1 << pl) - 1) >> pl;
+            s += mine ? it.y << pl : 0;
             e = s + (1 << pl) < e ? s + (1 << pl) : e;
-            todo = 1u;
+            todo = __ballot_sync(FULL, lane == 0 && mine);
         } else {
             const bool isshort = in && row_len <= kTailShort;
             if (sub == 0) {

@@ -169,3 +169,41 @@ def test_batch_of_every_kind(dev):
         for y, want in zip(ys, wants):
             assert np.array_equal(y.cpu().numpy().astype(np.float64), want)
             y.fill_(float("nan"))
+
+
+def test_shown_workspace_may_be_written(dev):
+    """The library's own workspace serves calls without one, whatever a caller
+    that asked for its address left in it (here a batch by tiles, whose header
+    counts dirty tiles where the row blocks count their lists)."""
+    from paper_1504_06474_gb300 import ssspmv as C
+    st = torch.cuda.Stream(dev)
+    m = 5000
+    rp, col, val, x = _matrix("uneven", m, 517, seed=9)
+    rpd, cd, vd, xd = _device(dev, (rp, col, val, x))
+    y = torch.empty(m, dtype=torch.float64, device=dev)
+    rq, colq, valq, xq = _matrix("oversized", m, 517, seed=10)
+    arrays = _device(dev, (rq, colq, valq, xq))
+    want = oracle.spmv(rq, colq, valq, xq)
+    y32, v32, x32 = torch.empty(m, device=dev), vd.float(), xd.float()
+    desc = torch.frombuffer(bytearray(C.batch_descriptors(
+        [(m, 517, int(rp[-1]), rpd, cd, v32, x32, y32)])), dtype=torch.uint8).to(dev)
+    opts = C.make_opts(W=15, variant=C.VARIANT_SPECULATIVE)
+    torch.cuda.synchronize()
+    C.check(C.ssspmv_csr_f64(m, 517, int(rp[-1]), rpd, cd, vd, xd, y, stream=st), "csr")
+    need = C.ssspmv_batched_workspace_bytes(1, int(rp[-1]), opts=opts)
+    big = np.arange(0, 2_000_001, 4, dtype=np.int32)  # a matrix that grows it enough
+    bm, bz = big.size - 1, int(big[-1])
+    grow = (torch.as_tensor(big, device=dev), torch.zeros(bz, dtype=torch.int32, device=dev),
+            torch.zeros(bz, dtype=torch.float64, device=dev), xd,
+            torch.empty(bm, dtype=torch.float64, device=dev))
+    torch.cuda.synchronize()
+    C.check(C.ssspmv_csr_f64(bm, 517, bz, *grow, stream=st), "grow")
+    ptr, size = C.ssspmv_cached_workspace(st)
+    assert size >= need
+    for _ in range(2):
+        C.check(C.ssspmv_csr_batched_f32(1, desc, int(rp[-1]), opts=opts, workspace=ptr,
+                                         ws_bytes=size, stream=st), "batched")
+        C.check(C.ssspmv_csr_f64(m, 517, int(rq[-1]), *arrays, y, stream=st), "csr")
+        st.synchronize()
+        assert np.array_equal(y.cpu().numpy(), want)
+    C.ssspmv_release_workspaces()
