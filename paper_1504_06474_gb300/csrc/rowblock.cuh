@@ -59,16 +59,22 @@ __host__ __device__ inline RowShape row_shape(int32_t m, int32_t nnz, int32_t va
     const int64_t mm = m > 0 ? m : 1;
     // one lane per row up to 27 entries on average (a 27-point stencil's 864
     // entries per group just fit), then 14 to 27 entries per lane; and more
-    // lanes where the groups would be too few to keep every warp busy (uniform
-    // rows of 0..40 entries, 120,007 of them, FP64: 24 us with two lanes, 27
-    // with one).  In FP32 far fewer groups are left whole, because the matrices
-    // of a batch share the GPU: 96 mixed ones take 297 to 317 us below 1,536
-    // groups, 397 with FP64's rule, and single small ones are as fast
-    const int64_t few = val_bytes == 8 ? 6144 : 384;
+    // lanes where the groups would be too few to keep every warp busy, if each
+    // lane still gets enough entries: FP64 above 6 up to 1,024 groups, above 8
+    // below 4,096.  Against 4 below 6,144 groups: bands, blocks and stencils of
+    // 7,000 to 40,000 rows 9 to 11 us -> 7 to 9, R-MAT scale 16 27 to 29 -> 19
+    // to 22 (the tiles: 25 to 27); whole groups from 1,536 on would make blocks
+    // of 92 entries per row (27,000 rows) 18 us instead of 14.5 and rows of
+    // 0..40 (120,007, axpby) 25.5 instead of 23.  In FP32 far fewer groups are
+    // left whole, because the matrices of a batch share the GPU: 96 mixed ones
+    // take 297 us below 384 groups, 317 below 1,536, 397 below 6,144, and
+    // single small ones are as fast.
     s.gs = 0;
     while (s.gs < 5 && (int64_t)nnz > ((int64_t)27 << s.gs) * mm) ++s.gs;
-    while (s.gs < 5 && (mm >> (5 - s.gs)) < few && (int64_t)nnz > ((int64_t)8 << s.gs) * mm)
-        ++s.gs;
+    auto split = [&](int64_t below, int64_t entries) {
+        return s.gs < 5 && (mm >> (5 - s.gs)) < below && (int64_t)nnz > (entries << s.gs) * mm;
+    };
+    while (val_bytes == 8 ? split(1025, 12) || split(4096, 16) : split(384, 8)) ++s.gs;
     // four groups at a time, where that leaves enough units for every warp
     // (half as many where several groups share a copy)
     const int64_t group = ((int64_t)nnz << (5 - s.gs)) / mm;  // its mean entries
