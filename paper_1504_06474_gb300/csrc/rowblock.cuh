@@ -22,11 +22,11 @@
 // lanes instead (a segmented sum inside the group).
 //
 // Measured (us a call among others; before: the three kernels of segsum.cuh).
-// FP64: 27-point stencil 160^3 272 -> 241 (the FP64 pipe alone needs 207), R-MAT
-// scale 22 with a 10^6-entry row 404 -> 330, banded half-width 31 (300,001 rows,
-// plan) 64 -> 51, uniform rows of 0..40 entries (120,007 rows, axpby) 43 -> 23,
-// rows of 1..8 entries and three of 500,000 91 -> 65, uniform 4096 rows 15 -> 7.
-// FP32: stencil 101x97x103 62 -> 45, R-MAT scale 20 110 -> 91, 96 mixed matrices
+// FP64: 27-point stencil 160^3 272 -> 239 (the FP64 pipe alone needs 207), R-MAT
+// scale 22 with a 10^6-entry row 402 -> 327, banded half-width 31 (300,001 rows,
+// plan) 64 -> 51, uniform rows of 0..40 entries (120,007 rows, axpby) 40 -> 22,
+// rows of 1..8 entries and three of 500,000 92 -> 62, uniform 4096 rows 15 -> 7.
+// FP32: stencil 101x97x103 62 -> 46, R-MAT scale 20 106 -> 89, 96 mixed matrices
 // 520 -> 337; BF16 values: stencil 120x125x131 110 -> 71.
 #pragma once
 #include <cstdint>

@@ -36,7 +36,13 @@ struct F64 {
     // R-MAT scale 22 kernel (b) 362 -> 350 us; the FP32 forms lose 2-3%)
     static constexpr bool kEarlyLongScan = true;
     static constexpr int kShortRowWarps = 14;  // short rows: keep L1 for the gathers (measured)
-    static constexpr int kRowWarps = 20;  // row blocks: warps per block (96 registers)
+    // row blocks: warps per block (96 registers).  The smallest stages of 19
+    // warps take 160 KB of shared memory, those of 20 168, past the carve-out
+    // that leaves 92 KB of L1 instead of 60: rows of 1..8 entries 48.6 -> 46.5
+    // us, axpby of rows of 0..40 24.3 -> 23.3, R-MAT scale 22 116 -> 113 (rows
+    // of 0..20: 55 -> 57; 18 warps: 116 for the R-MAT, 22 with 80 registers:
+    // 119, and stencil 160^3 245 instead of 239)
+    static constexpr int kRowWarps = 19;
     static constexpr int kLaneBatch = 4, kSplitBatch = 4;  // gathers in flight per lane
     // row blocks: a group of T entries whose longest lane takes n steps keeps
     // a lane per row (or G lanes) rather than an even split of its entries
