@@ -605,6 +605,7 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
             }
             if (!mbar_wait_bounded(&sc->bar, phase)) {
                 if (lane == 0) atomicOr(a.head + kWordErr, SSSPMV_DEV_TIMEOUT);
+                mbar_wait_bounded(&sc->bar, phase);  // once more before the stage goes
                 return;
             }
             phase ^= 1u;
