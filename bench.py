@@ -63,8 +63,8 @@ def peaks():
 # the sources that define the product's kernels and their launches (device code,
 # tile and row-block shapes, workspace carve-up); host-only files do not change
 # their traffic
-KERNEL_B_SOURCES = ("layout.h", "launch.cuh", "ptx.cuh", "rowblock.cuh", "segsum.cuh",
-                    "spmv_f64.cu")
+KERNEL_B_SOURCES = ("layout.h", "launch.cuh", "ptx.cuh", "rowblock.cuh", "rowshape.h",
+                    "segsum.cuh", "spmv_f64.cu")
 
 
 def product_path(opts_kw: dict) -> dict:

@@ -16,7 +16,7 @@ LIB = os.path.join(PKG, "libssspmv.so")
 
 SOURCES = ["api.cu", "partition.cu", "spmv_f64.cu", "spmv_f32.cu", "spmv_bf16.cu", "batched.cu",
            "rows.cu", "mlp.cu", "noalloc.cu", "range.cu"]
-HEADERS = ["ptx.cuh", "segsum.cuh", "launch.cuh", "rowblock.cuh", "layout.h"]
+HEADERS = ["ptx.cuh", "segsum.cuh", "launch.cuh", "rowblock.cuh", "rowshape.h", "layout.h"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
