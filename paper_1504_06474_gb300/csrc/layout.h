@@ -26,7 +26,8 @@ inline int32_t auto_bunch_tiles(int64_t ntiles)
 }
 
 // The words at the front of a workspace (uint32 each):
-//   [0] device error bits          cleared by kernel (a)
+//   [0] device error bits          cleared by kernel (a); by row blocks written
+//                                  by rowtail_kernel
 //   [1] bunch ticket of kernel (b) cleared by kernel (a)
 //   [2] dirty-tile count           cleared by kernel (a); kernel (b) appends
 //                                  the dirty tiles it leaves to kernel (c)
@@ -34,12 +35,14 @@ inline int32_t auto_bunch_tiles(int64_t ntiles)
 //                                  empty rows, cleared by kernel (c)
 //   [4,5] lengths of the lists of rows rowblock_kernel leaves to
 //         rowtail_kernel, [6] rowtail_kernel's ticket, [7] its finished
-//         blocks, [8] rowblock_kernel's ticket: zero between calls
+//         blocks, [8] rowblock_kernel's ticket, [9] its error bits, which
+//         rowtail_kernel moves to word 0: zero between calls
 //         (rowtail_kernel clears them)
 // (a plan execution, which skips kernel (a), clears words 0..2 and keeps the
 // plan's flag)
 constexpr int kWordErr = 0, kWordTicket = 1, kWordDirty = 2, kWordSpread = 3;
-constexpr int kWordLists = 4, kWordTailTicket = 6, kWordTailDone = 7, kWordUnitTicket = 8;
+constexpr int kWordLists = 4, kWordTailTicket = 6, kWordTailDone = 7, kWordUnitTicket = 8,
+              kWordRowErr = 9;
 constexpr size_t kHeaderBytes = 64;
 
 struct Layout {

@@ -230,7 +230,7 @@ static __device__ __noinline__ void list_group(const RowArgs &a, int32_t mat, in
     if ((uint64_t)rbase + __popc(leads) > (uint32_t)a.max_ranges ||
         (uint64_t)pbase + (uint32_t)total > (uint32_t)a.max_pieces) {
         // more than any valid row_ptr can list
-        if (lane == 0) atomicOr(a.head + kWordErr, SSSPMV_DEV_RANGE);
+        if (lane == 0) atomicOr(a.head + kWordRowErr, SSSPMV_DEV_RANGE);
         return;
     }
     if (lead) {
@@ -324,7 +324,6 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
     __syncthreads();
     grid_dep_wait();  // everything read below may come from the kernel before
     grid_dep_trigger();
-    if (!BATCHED && blockIdx.x == 0 && threadIdx.x == 0) a.head[kWordErr] = 0u;
 
     // the current unit's matrix (in a batch: loaded again when it changes)
     const X *__restrict__ x = static_cast<const X *>(a.x);
@@ -513,7 +512,7 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
                 }
             }
             if (!mbar_wait_bounded(&sc->bar, phase)) {
-                if (lane == 0) atomicOr(a.head + kWordErr, SSSPMV_DEV_TIMEOUT);
+                if (lane == 0) atomicOr(a.head + kWordRowErr, SSSPMV_DEV_TIMEOUT);
                 mbar_wait_bounded(&sc->bar, phase);  // once more before the stage goes
                 return;
             }
@@ -652,7 +651,15 @@ __global__ void __launch_bounds__(kTailThreads, BLOCKS) rowtail_kernel(const Row
     grid_dep_wait();
     uint32_t nr = *(volatile const uint32_t *)(a.head + kWordLists);
     uint32_t np = *(volatile const uint32_t *)(a.head + kWordLists + 1);
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.head[kWordUnitTicket] = 0u;  // (r1)'s
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.head[kWordUnitTicket] = 0u;  // (r1)'s
+        // (r1)'s error bits become the call's (beside a batch's set-up's).  They
+        // have a word of their own because no block of (r1) could clear the
+        // call's word before all the others may set a bit in it.
+        const uint32_t bits = *(volatile const uint32_t *)(a.head + kWordRowErr);
+        a.head[kWordErr] = BATCHED ? a.head[kWordErr] | bits : bits;
+        a.head[kWordRowErr] = 0u;
+    }
     if (nr + np == 0u) return;  // every row was staged
     // (an invalid row_ptr may have been refused more than the lists hold)
     nr = nr > (uint32_t)a.max_ranges ? 0u : nr;

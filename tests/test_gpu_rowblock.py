@@ -207,3 +207,27 @@ def test_shown_workspace_may_be_written(dev):
         st.synchronize()
         assert np.array_equal(y.cpu().numpy(), want)
     C.ssspmv_release_workspaces()
+
+
+@pytest.mark.parametrize("kind", ["upto4", "oversized"])
+def test_error_bits_of_the_first_kernel_reach_the_status(dev, kind):
+    """A bit that a block of the first kernel sets (word 9 of the workspace, here
+    set before the call) is the call's status whichever block runs first, with
+    rows left to the second kernel and without, and gone after the next call."""
+    from paper_1504_06474_gb300 import ssspmv as C
+    m = 9001
+    rp, col, val, x = _matrix(kind, m, 517, seed=3)
+    nnz, want = int(rp[-1]), oracle.spmv(rp, col, val, x)
+    rpd, cd, vd, xd = _device(dev, (rp, col, val, x))
+    ws = torch.empty(C.ssspmv_workspace_bytes(m, nnz, 8, None), dtype=torch.uint8, device=dev)
+    y = torch.empty(m, dtype=torch.float64, device=dev)
+    plan = C.ssspmv_plan_create(m, 517, nnz, rpd, 8, workspace=ws)
+    try:
+        for bits in (0, C.SSSPMV_DEV_RANGE, 0, C.SSSPMV_DEV_TIMEOUT, 0):
+            if bits:
+                ws[36:40].view(torch.int32).fill_(bits)
+            C.check(C.ssspmv_plan_execute(plan, cd, vd, xd, y), "execute")
+            assert C.ssspmv_device_status(ws) == bits
+            assert np.array_equal(y.cpu().numpy(), want)
+    finally:
+        C.ssspmv_plan_destroy(plan)
