@@ -970,10 +970,15 @@ int run_rowblock(const Call &c)
     int rc = a.shape.gs > 0 ? launch_rowblock<P, true>(c, a) : launch_rowblock<P, false>(c, a);
     if (rc) return rc;
     if (c.ev && (e = cudaEventRecord(c.ev[2], c.stream)) != cudaSuccess)
-        return record_cuda_error(e);
+        rc = record_cuda_error(e);
     // small matrices: fewer, longer rounds of loads per row
-    rc = c.nnz < kTailWide ? launch_rowtail<P, 8, 2>(c, a) : launch_rowtail<P, 4, 3>(c, a);
-    if (rc) return rc;
+    if (!rc) rc = c.nnz < kTailWide ? launch_rowtail<P, 8, 2>(c, a) : launch_rowtail<P, 4, 3>(c, a);
+    if (rc) {
+        // (r1) has run and (r2) will not (its first launch loads it, and may find
+        // no memory): the counters (r1) leaves must not meet the next call
+        (void)cudaMemsetAsync(a.head, 0, kHeaderBytes, c.stream);
+        return rc;
+    }
     if (c.ev && (e = cudaEventRecord(c.ev[3], c.stream)) != cudaSuccess)
         return record_cuda_error(e);
     e = cudaGetLastError();
