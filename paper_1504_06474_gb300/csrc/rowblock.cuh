@@ -301,6 +301,27 @@ __device__ __forceinline__ int32_t inside(int32_t p, int32_t b, int32_t e)
     return p < b ? b : (p > e ? e : p);
 }
 
+// the matrix that unit u of a batch belongs to: the last one of `count` that
+// starts at or before it, `from` or a later one (all lanes call it).  The next
+// 32 at once, then a search by 33 ways: a walk from one record to the next, which
+// every warp makes past every matrix, took 2,198 us of 10,000 matrices of 1,000
+// entries and 225 of 1,000 of 10,000; so 195 and 76 (the tiles: 188 and 66; 96
+// mixed matrices: 336 us either way).
+__device__ __forceinline__ int32_t find_matrix(const RowMat *mats, int32_t count, int32_t from,
+                                               int32_t u)
+{
+    const int lane = threadIdx.x & 31;
+    int32_t lo = from, hi = count, step = 1;
+    while (hi - lo > 1) {
+        const int32_t i = lo + (lane + 1) * step;
+        const int n = __popc(__ballot_sync(FULL, i < hi && __ldg(&mats[i].unit_base) <= u));
+        lo += n * step;
+        if (n < 32 && lo + step < hi) hi = lo + step;
+        step = (hi - lo + 31) >> 5;
+    }
+    return lo;
+}
+
 template <class P, bool MULTI, bool BATCHED = false>
 __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32, 1)
     rowblock_kernel(const RowArgs a, int32_t stage_bytes, int32_t col_off)
@@ -385,7 +406,7 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
         int32_t u = (int32_t)t, um = m, ugs = gs, us = a.shape.us, nbig = a.nbig;
         const int32_t *row_ptr = a.row_ptr;
         if constexpr (BATCHED) {
-            while (at_mat + 1 < a.count && u >= __ldg(&a.mats[at_mat + 1].unit_base)) ++at_mat;
+            at_mat = find_matrix(a.mats, a.count, at_mat, u);
             const RowMat *mm = a.mats + at_mat;
             row_ptr = ldg_ptr(&mm->row_ptr);
             um = __ldg(&mm->m);

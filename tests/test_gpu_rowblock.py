@@ -231,3 +231,73 @@ def test_error_bits_of_the_first_kernel_reach_the_status(dev, kind):
             assert np.array_equal(y.cpu().numpy(), want)
     finally:
         C.ssspmv_plan_destroy(plan)
+
+
+def _small_matrices(dev, count, seed):
+    """A batch of `count` small matrices over one x (rows of 0 to 15 entries, some
+    matrices without rows or entries): descriptors, all y in a row, the sum of
+    nnz, and what y has to be."""
+    rng = np.random.default_rng(seed)
+    n = 517
+    ms = rng.integers(20, 120, size=count)
+    ms[rng.random(count) < 0.1] = 0
+    ms[-3:] = 0
+    lens = rng.integers(0, 16, size=int(ms.sum()))
+    row0 = np.concatenate([[0], np.cumsum(ms)])
+    lens[row0[count // 3]:row0[count // 3 + 2]] = 0
+    nnz = np.array([lens[a:b].sum() for a, b in zip(row0[:-1], row0[1:])])
+    at = np.concatenate([[0], np.cumsum((nnz + 3) // 4 * 4)])  # 16-byte aligned starts
+    col = rng.integers(0, n, size=int(at[-1]) + 4).astype(np.int32)
+    val = rng.integers(-6, 7, size=int(at[-1]) + 4).astype(np.float32)
+    x = rng.integers(-6, 7, size=n).astype(np.float32)
+    rps = [np.concatenate([[0], np.cumsum(lens[a:b])]) for a, b in zip(row0[:-1], row0[1:])]
+    used = np.concatenate([np.arange(k) + a for k, a in zip(nnz, at)]).astype(np.int64)
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    want = oracle.spmv(rp, col[used], val[used].astype(float), x.astype(float))
+    rpd, cd, vd, xd = _device(dev, (np.concatenate(rps).astype(np.int32), col, val, x))
+    y = torch.full((int(row0[-1]),), float("nan"), device=dev)
+    rec = np.zeros(count, dtype=[("m", "<i4"), ("n", "<i4"), ("nnz", "<i4"), ("reserved", "<i4"),
+                                 ("rp", "<u8"), ("col", "<u8"), ("val", "<u8"), ("x", "<u8"),
+                                 ("y", "<u8")])
+    rec["m"], rec["n"], rec["nnz"] = ms, n, nnz
+    rec["rp"] = rpd.data_ptr() + 4 * (row0[:-1] + np.arange(count))
+    rec["col"], rec["val"] = cd.data_ptr() + 4 * at[:-1], vd.data_ptr() + 4 * at[:-1]
+    rec["x"], rec["y"] = xd.data_ptr(), y.data_ptr() + 4 * row0[:-1]
+    desc = torch.as_tensor(np.frombuffer(rec.tobytes(), np.uint8).copy(), device=dev)
+    return desc, y, int(nnz.sum()), want, (rpd, cd, vd, xd)
+
+
+@pytest.mark.parametrize("count", [31, 32, 33, 34, 1057, 8000])
+def test_batch_finds_the_matrix_of_every_unit(dev, count):
+    from paper_1504_06474_gb300 import ssspmv as C
+    desc, y, total, want, keep = _small_matrices(dev, count, seed=count)
+    ws = torch.empty(C.ssspmv_batched_workspace_bytes(count, total), dtype=torch.uint8, device=dev)
+    C.check(C.ssspmv_csr_batched_f32(count, desc, total, workspace=ws), "batched")
+    assert C.ssspmv_device_status(ws) == 0
+    assert np.array_equal(y.cpu().numpy().astype(np.float64), want)
+
+
+def _us(fn, reps=7):
+    times = []
+    for i in range(reps + 2):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        fn()
+        b.record()
+        b.synchronize()
+        times.append(a.elapsed_time(b) * 1e3)
+    return float(np.median(times[2:]))
+
+
+def test_many_matrices_are_no_slower_than_by_tiles(dev):
+    # (walking past every matrix, each warp took ten times as long as the tiles)
+    from paper_1504_06474_gb300 import ssspmv as C
+    count = 8000
+    desc, y, total, want, keep = _small_matrices(dev, count, seed=1)
+    us = []
+    for opts in (None, C.make_opts(W=15, variant=C.VARIANT_SPECULATIVE)):
+        ws = torch.empty(C.ssspmv_batched_workspace_bytes(count, total, 4, opts),
+                         dtype=torch.uint8, device=dev)
+        us.append(_us(lambda: C.check(C.ssspmv_csr_batched_f32(count, desc, total, opts=opts,
+                                                               workspace=ws), "batched")))
+    assert us[0] <= 1.5 * us[1], us
