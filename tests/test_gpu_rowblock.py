@@ -301,3 +301,57 @@ def test_many_matrices_are_no_slower_than_by_tiles(dev):
         us.append(_us(lambda: C.check(C.ssspmv_csr_batched_f32(count, desc, total, opts=opts,
                                                                workspace=ws), "batched")))
     assert us[0] <= 1.5 * us[1], us
+
+
+# several lanes per row and four groups at a time (the sizes are checked on the
+# CPU in test_rowshape_host.py): kind, m, lanes per row
+LANES = [("const28", 400_003, 2), ("upto56", 400_003, 2), ("const60", 200_003, 4),
+         ("upto120", 200_003, 4), ("const120", 100_003, 8), ("upto240", 100_003, 8),
+         ("const220", 50_003, 16), ("upto440", 50_003, 16), ("const440", 25_003, 32),
+         ("upto900", 25_003, 32)]
+
+
+@pytest.mark.parametrize("kind,m,lanes,prec",
+                         [c + ("f64",) for c in LANES] +
+                         [c + (p,) for c in LANES[1::2] for p in ("f32", "bf16")])
+def test_several_lanes_per_row_in_units_of_four_groups(dev, kind, m, lanes, prec):
+    from paper_1504_06474_gb300 import ssspmv as C
+    rp, col, val, x = _matrix(kind, m, 517, seed=lanes)
+    if kind.startswith("upto"):  # and a run of empty rows across units
+        gone = slice(m // 3, m // 3 + 300)
+        lens = np.diff(rp)
+        lens[gone] = 0
+        rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        col, val = col[: rp[-1]], val[: rp[-1]]
+    nnz, want = int(rp[-1]), oracle.spmv(rp, col, val, x)
+    vt = {"f64": torch.float64, "f32": torch.float32, "bf16": torch.bfloat16}[prec]
+    fn = {"f64": C.ssspmv_csr_f64, "f32": C.ssspmv_csr_f32, "bf16": C.ssspmv_csr_bf16f32}[prec]
+    rpd, cd, vd, xd = _device(dev, (rp, col, val, x))
+    vd, xt = vd.to(vt), torch.float64 if prec == "f64" else torch.float32
+    if prec == "bf16":
+        vd = vd.view(torch.int16)
+    y = torch.full((m,), float("nan"), dtype=xt, device=dev)
+    C.check(fn(m, 517, nnz, rpd, cd, vd, xd.to(xt), y), prec)
+    assert np.array_equal(y.cpu().numpy().astype(np.float64), want)
+
+
+def test_several_lanes_per_row_in_a_batch(dev):
+    from paper_1504_06474_gb300 import ssspmv as C
+    keep, descs, wants, ys = [], [], [], []
+    for i, (kind, m) in enumerate([("upto12", 700), ("upto120", 200_003), ("empty", 33),
+                                   ("upto900", 25_003), ("pieces", 5000), ("upto56", 400_003)]):
+        rp, col, val, x = _matrix(kind, m, 517, seed=200 + i)
+        rpd, cd, vd, xd = _device(dev, (rp, col, val.astype(np.float32), x.astype(np.float32)))
+        y = torch.full((m,), float("nan"), dtype=torch.float32, device=dev)
+        keep.append((rpd, cd, vd, xd))
+        descs.append((m, 517, int(rp[-1]), rpd, cd, vd, xd, y))
+        wants.append(oracle.spmv(rp, col, val, x))
+        ys.append(y)
+    total = sum(d[2] for d in descs)
+    desc = torch.frombuffer(bytearray(C.batch_descriptors(descs)), dtype=torch.uint8).to(dev)
+    ws = torch.empty(C.ssspmv_batched_workspace_bytes(len(descs), total), dtype=torch.uint8,
+                     device=dev)
+    C.check(C.ssspmv_csr_batched_f32(len(descs), desc, total, workspace=ws), "batched")
+    assert C.ssspmv_device_status(ws) == 0
+    for y, want in zip(ys, wants):
+        assert np.array_equal(y.cpu().numpy().astype(np.float64), want)

@@ -18,6 +18,17 @@ using namespace ssspmv;
 extern "C" {
 int32_t pieces(int32_t len, int32_t pl) { return row_pieces(len, pl); }
 int32_t end_of(int32_t s, int32_t e, int32_t pl) { return piece_end(s, e, pl); }
+void shape(int32_t m, int32_t nnz, int32_t val_bytes, int32_t *out)
+{
+    const RowShape s = row_shape(m, nnz, val_bytes);
+    const RowUnits u = row_units(m, s);
+    out[0] = s.gs;
+    out[1] = s.us;
+    out[2] = s.cap;
+    out[3] = s.piece;
+    out[4] = u.nbig;
+    out[5] = u.nunits;
+}
 }
 """
 
@@ -55,3 +66,32 @@ def test_no_entries_no_pieces(lib, pl):
     for n in (0, -1, -2048, -(2**31) + 1):
         assert lib.pieces(n, pl) == 0
     assert lib.end_of(MAX_DIM, MAX_DIM, pl) == MAX_DIM
+
+
+def _shape(lib, m, nnz, val_bytes):
+    out = (ctypes.c_int32 * 6)()
+    lib.shape(m, nnz, val_bytes, out)
+    return dict(zip(("gs", "us", "cap", "piece", "nbig", "nunits"), out))
+
+
+def test_the_gpu_cases_take_the_shapes_they_are_for(lib):
+    from test_gpu_rowblock import LANES
+    for kind, m, lanes in LANES:
+        nnz = m * int(kind[5:]) if kind.startswith("const") else m * int(kind[4:]) // 2
+        for val_bytes in (8, 4, 2):
+            s = _shape(lib, m, nnz, val_bytes)
+            assert (1 << s["gs"], s["us"]) == (lanes, 2), (kind, val_bytes, s)
+            assert 0 < s["nbig"] < s["nunits"]
+
+
+def test_units_cover_the_rows(lib):
+    for m in (1, 31, 32, 33, 127, 9001, 400_003, 2_000_000_011, MAX_DIM):
+        for mean in (0, 1, 10, 28, 60, 440):
+            nnz = min(m * mean, MAX_DIM)
+            for val_bytes in (8, 4, 2):
+                s = _shape(lib, m, nnz, val_bytes)
+                rows = 32 >> s["gs"]
+                single = s["nunits"] - s["nbig"]
+                covered = s["nbig"] * (rows << s["us"]) + single * rows
+                assert 0 <= covered - m < rows, (m, mean, s)
+                assert s["cap"] % 8 == 0
