@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(kPrepThreads)
             continue;
         }
         nt += ((int64_t)d.nnz + L - 1) / L;
-        nu += row_units(d.m, row_shape(d.m, d.nnz, 4)).nunits;
+        nu += row_units(d.m, d.nnz, row_shape(d.m, d.nnz, 4)).nunits;
     }
     if (bad) atomicOr(head + kWordErr, SSSPMV_DEV_BATCH);
     int64_t tot_t = 0, tot_u = 0;
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kPrepThreads)
         if (!valid_desc(d) || !fits)
             d = DescView{0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, nullptr};
         const RowShape s = row_shape(d.m, d.nnz, 4);
-        const RowUnits u = row_units(d.m, s);
+        const RowUnits u = row_units(d.m, d.nnz, s);
         RowMat r;
         r.val = d.val;
         r.col = d.col;

@@ -488,6 +488,12 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
                     jn += rows;
                 }
             }
+            if (!BATCHED && te == ts) {  // rows without entries: nothing to copy
+                for (int32_t k = j + lane; k < jn; k += 32)
+                    if (cur.r0 + k < m) store(cur.r0 + k, P::zero());
+                j = jn;
+                continue;
+            }
             __syncwarp();  // every lane is done with the copy before
             stage_copy(st, col_off, &sc->bar, val, col, nnz, ts, te, pol_stream);
             if (nxt.nr < 0) nxt = next_unit();
@@ -982,7 +988,7 @@ int run_rowblock(const Call &c)
     a.max_pieces = (int32_t)rl.pieces;
     a.m = c.m;
     a.nnz = c.nnz;
-    const RowUnits units = row_units(c.m, a.shape);
+    const RowUnits units = row_units(c.m, c.nnz, a.shape);
     a.nbig = units.nbig;
     a.nunits = units.nunits;
     a.alpha = c.alpha;

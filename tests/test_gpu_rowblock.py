@@ -355,3 +355,36 @@ def test_several_lanes_per_row_in_a_batch(dev):
     assert C.ssspmv_device_status(ws) == 0
     for y, want in zip(ys, wants):
         assert np.array_equal(y.cpu().numpy().astype(np.float64), want)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("share", [0.0, 1e-6, 0.001, 0.5])
+def test_many_rows_of_hardly_any_entries(dev, share, prec):
+    """Units without entries (nothing is copied), alone and between others, up to
+    a matrix without any; NaN beforehand shows a row that is not written."""
+    from paper_1504_06474_gb300 import ssspmv as C
+    rng = np.random.default_rng(4)
+    m, n = 2_500_003, 517
+    lens = (rng.random(m) < share) * rng.integers(1, 3, size=m)
+    lens[400_000:900_000] = 0
+    lens[700_001:700_400] = 3 if share else 0
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    nnz = int(rp[-1])
+    col = rng.integers(0, n, size=nnz).astype(np.int32)
+    val = rng.integers(-6, 7, size=nnz).astype(float)
+    x = rng.integers(-6, 7, size=n).astype(float)
+    want = oracle.spmv(rp, col, val, x)
+    vt = {"f64": torch.float64, "f32": torch.float32, "bf16": torch.bfloat16}[prec]
+    fn = {"f64": C.ssspmv_csr_f64, "f32": C.ssspmv_csr_f32, "bf16": C.ssspmv_csr_bf16f32}[prec]
+    rpd, cd, vd, xd = _device(dev, (rp, col, val, x))
+    xt = torch.float64 if prec == "f64" else torch.float32
+    vd = vd.to(vt).view(torch.int16) if prec == "bf16" else vd.to(vt)
+    y = torch.full((m,), float("nan"), dtype=xt, device=dev)
+    C.check(fn(m, n, nnz, rpd, cd, vd, xd.to(xt), y), prec)
+    assert np.array_equal(y.cpu().numpy().astype(np.float64), want)
+    if prec == "f64":  # y = 2 A x + 3 y: rows without entries are scaled too
+        C.check(C.ssspmv_csr_f64_axpby(m, n, nnz, rpd, cd, vd, xd, y, 2.0, 3.0), "axpby")
+        assert np.array_equal(y.cpu().numpy(), 5.0 * want)
+        y.fill_(1.0)
+        C.check(C.ssspmv_csr_f64_axpby(m, n, nnz, rpd, cd, vd, xd, y, 2.0, 3.0), "axpby")
+        assert np.array_equal(y.cpu().numpy(), 2.0 * want + 3.0)

@@ -21,7 +21,7 @@ int32_t end_of(int32_t s, int32_t e, int32_t pl) { return piece_end(s, e, pl); }
 void shape(int32_t m, int32_t nnz, int32_t val_bytes, int32_t *out)
 {
     const RowShape s = row_shape(m, nnz, val_bytes);
-    const RowUnits u = row_units(m, s);
+    const RowUnits u = row_units(m, nnz, s);
     out[0] = s.gs;
     out[1] = s.us;
     out[2] = s.cap;
@@ -95,3 +95,11 @@ def test_units_cover_the_rows(lib):
                 covered = s["nbig"] * (rows << s["us"]) + single * rows
                 assert 0 <= covered - m < rows, (m, mean, s)
                 assert s["cap"] % 8 == 0
+
+
+def test_short_rows_are_few_units(lib):
+    # (a unit costs some 2 us of a warp's time however little it holds)
+    for m, mean, most in ((20_000_000, 1, 161_000), (20_000_000, 3, 161_000),
+                          (20_000_000, 20, 185_000), (2_000_000, 1, 20_500)):
+        s = _shape(lib, m, m * mean, 8)
+        assert s["us"] == 2 and s["nunits"] <= most, (m, mean, s)
