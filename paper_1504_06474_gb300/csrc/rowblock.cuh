@@ -80,22 +80,21 @@ struct RowArgs {
 // ---------------------------------------------------------------------------
 
 // entry loop of one lane: n entries, the i-th at shared index i * G (G == 0:
-// i * stride); every lane has nmin or more, none more than nmax.  ROT: the lane
-// starts at its rot-th entry and wraps around (rot <= n).  A multiply-add that
+// i * stride), added to acc; every lane has nmin or more, none more than nmax.
+// ROT: the lane starts at its rot-th entry and wraps around (rot <= n).  A multiply-add that
 // no lane needs is branched over: with every lane predicated off it
 // would still hold the FP64 pipe for its 76 cycles (measured).
 template <class P, int UN, int G, bool ROT>
 __device__ __forceinline__ typename P::acc_t lane_dot(const typename P::val_t *vs,
                                                       const int32_t *cs,
                                                       const typename P::x_t *x, int n, int nmin,
-                                                      int nmax, int stride, int rot, uint64_t pol)
+                                                      int nmax, int stride, int rot, uint64_t pol,
+                                                      typename P::acc_t acc)
 {
     using X = typename P::x_t;
-    using A = typename P::acc_t;
     const int st = G > 0 ? G : stride;
     // shared index of the lane's i-th entry
     auto at = [&](int i) { return ROT ? (i + rot < n ? i + rot : i + rot - n) * st : i * st; };
-    A acc = P::zero();
     int i = 0;
     for (; i + UN <= nmin; i += UN) {
         X xv[UN];
@@ -462,7 +461,7 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
         while (j < cur.nr) {
             const int32_t g0 = inside(rp[j], b, e), ge = inside(rp[j + rows], g0, e);
             const int32_t T = ge - g0;
-            if (T > 2 * cap) {
+            if (T > 2 * cap && (!MULTI || T > row_most(nnz, gs, cap))) {
                 const int32_t l = lane < rows ? lane : 0;
                 const int32_t rs = inside(rp[j + l], g0, ge), re = inside(rp[j + l + 1], rs, ge);
                 const int32_t left = m - (cur.r0 + j);
@@ -508,6 +507,9 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
                         FULL, (unsigned)(MULTI ? (n + (1 << gs) - 1) >> gs : n));
                 }
                 even = P::rows_even(steps, te - ts);
+            } else if (MULTI && rows == 1) {
+                steps = (te - ts + 31) >> 5;
+                even = true;  // a part of one long row
             }
             const int32_t Tp = te - ts;
             const int32_t C = ((Tp + 31) >> 5) | 1;
@@ -566,10 +568,16 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
                     if (__popc(banks) <= 8 && nmax >= 8)
                         acc = lane_dot<P, P::kLaneBatch, MULTI ? 0 : 1, true>(
                             sv + first, scol + first, x, n, nmin, nmax, 1 << gs,
-                            n > 0 ? lrow % n : 0, pol_keep);
+                            n > 0 ? lrow % n : 0, pol_keep, MULTI ? carry : P::zero());
                     else
                         acc = lane_dot<P, P::kLaneBatch, MULTI ? 0 : 1, false>(
-                            sv + first, scol + first, x, n, nmin, nmax, 1 << gs, 0, pol_keep);
+                            sv + first, scol + first, x, n, nmin, nmax, 1 << gs, 0, pol_keep,
+                            MULTI ? carry : P::zero());
+                    if (MULTI && te < ge) {  // a part of one long row: lane by lane
+                        carry = acc;
+                        continue;
+                    }
+                    if (MULTI) carry = P::zero();
                     if (MULTI)
                         for (int d = 1; d < (1 << gs); d <<= 1)
                             acc = P::add(acc, P::shfl(acc, lane ^ d));

@@ -67,6 +67,23 @@ SSSPMV_HD inline RowShape row_shape(int32_t m, int32_t nnz, int32_t val_bytes)
     return s;
 }
 
+// Most entries of a group that (r1) works off itself, a stage at a time; larger
+// groups are listed.  Two stages, or, where a group is one row, as many as a
+// warp's share of the matrix has, up to eight: rows that are all this long would
+// nearly all be listed, a range of one row each or pieces of unlike lengths, and
+// (r2) takes one such list entry per chain of loads.  50 million entries in rows
+// of 2,100, two stages at most against this: FP64 197 us and 121 (the tiles 146),
+// FP32 178 and 86 (90), BF16 values 176 and 81 (100); of 5,000: 158 and 118
+// (165), 138 and 85 (111), 136 and 78 (100); of 900, two stages both times, but
+// lane by lane now instead of split evenly: 180 and 143 (146), 133 and 100 (90),
+// 133 and 99 (97).
+SSSPMV_HD inline int32_t row_most(int32_t nnz, int32_t gs, int32_t cap)
+{
+    const int32_t share = nnz >> 12;
+    if (gs < 5 || share <= 2 * cap) return 2 * cap;
+    return share < 8 * cap ? share : 8 * cap;
+}
+
 // bounds of the lists (r1) writes: at most one range of rows per `piece`
 // entries or part of it of an oversized group, and rows longer than a piece
 // cut into pieces

@@ -388,3 +388,80 @@ def test_many_rows_of_hardly_any_entries(dev, share, prec):
         y.fill_(1.0)
         C.check(C.ssspmv_csr_f64_axpby(m, n, nnz, rpd, cd, vd, xd, y, 2.0, 3.0), "axpby")
         assert np.array_equal(y.cpu().numpy(), 2.0 * want + 3.0)
+
+
+def _long_rows(seed):
+    """Rows of up to 7,200 entries, 24 million in all, so that rows of up to
+    about 5,860 are worked off in several stages and longer ones in pieces; at
+    the edges of stages (888), of both, and empty ones."""
+    rng = np.random.default_rng(seed)
+    lens = rng.integers(2500, 7200, size=5000)
+    lens[rng.choice(5000, 500, replace=False)] = 0
+    share = int(lens.sum()) >> 12
+    edges = [0, 1, 31, 32, 33, 887, 888, 889, 896, 1775, 1776, 1777, 2663, 2664, 2665, 2672,
+             share - 1, share, share + 1, 7104, 7105]
+    lens[1000: 1000 + len(edges)] = edges
+    lens[-1] = 3001
+    return np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "bf16"])
+def test_rows_of_several_stages(dev, prec):
+    from paper_1504_06474_gb300 import ssspmv as C
+    rng = np.random.default_rng(8)
+    n = 60_000
+    rp = _long_rows(8)
+    m, nnz = rp.size - 1, int(rp[-1])
+    col = rng.integers(0, n, size=nnz).astype(np.int32)
+    val, x = rng.integers(-6, 7, size=nnz).astype(float), rng.integers(-6, 7, size=n).astype(float)
+    want = oracle.spmv(rp, col, val, x)
+    vt = {"f64": torch.float64, "f32": torch.float32, "bf16": torch.bfloat16}[prec]
+    fn = {"f64": C.ssspmv_csr_f64, "f32": C.ssspmv_csr_f32, "bf16": C.ssspmv_csr_bf16f32}[prec]
+    xt = torch.float64 if prec == "f64" else torch.float32
+    rpd, cd, vd, xd = _device(dev, (rp, col, val, x))
+    vd = vd.to(vt).view(torch.int16) if prec == "bf16" else vd.to(vt)
+    y = torch.full((m,), float("nan"), dtype=xt, device=dev)
+    C.check(fn(m, n, nnz, rpd, cd, vd, xd.to(xt), y), prec)
+    assert np.array_equal(y.cpu().numpy().astype(np.float64), want)
+    if prec == "f32":  # the same bits in a batch
+        val32, x32 = (torch.as_tensor(rng.uniform(-1, 1, k).astype(np.float32), device=dev)
+                      for k in (nnz, n))
+        C.check(fn(m, n, nnz, rpd, cd, val32, x32, y), "f32")
+        yb = torch.full((m,), float("nan"), device=dev)
+        desc = torch.frombuffer(bytearray(C.batch_descriptors(
+            [(m, n, nnz, rpd, cd, val32, x32, yb)])), dtype=torch.uint8).to(dev)
+        ws = torch.empty(C.ssspmv_batched_workspace_bytes(1, nnz), dtype=torch.uint8, device=dev)
+        C.check(C.ssspmv_csr_batched_f32(1, desc, nnz, workspace=ws), "batched")
+        assert torch.equal(y, yb)
+    elif prec == "f64":
+        C.check(C.ssspmv_csr_f64_axpby(m, n, nnz, rpd, cd, vd, xd, y, 2.0, -3.0), "axpby")
+        assert np.array_equal(y.cpu().numpy(), -want)
+        val, x = rng.uniform(-1, 1, nnz), rng.uniform(-1, 1, n)
+        vd, xd = _device(dev, (val, x))
+        C.check(fn(m, n, nnz, rpd, cd, vd, xd, y), "f64")
+        yref, s = oracle.spmv_dot2(rp, col, val, x)
+        assert np.all(np.abs(y.cpu().numpy() - yref) <= 1e-13 * s)
+
+
+@pytest.mark.parametrize("prec,length", [("f32", 2100), ("bf16", 2100), ("f64", 2100),
+                                         ("f32", 900)])
+def test_long_rows_are_no_slower_than_by_tiles(dev, prec, length):
+    # (all listed, rows of 2,100 took 1.35 to twice the tiles' time)
+    from paper_1504_06474_gb300 import ssspmv as C
+    m, n = 25_000_000 // length, 100_000
+    nnz = m * length
+    rp = torch.arange(m + 1, device=dev, dtype=torch.int32) * length
+    col = (torch.arange(nnz, device=dev) % n).to(torch.int32)
+    vt = {"f64": torch.float64, "f32": torch.float32, "bf16": torch.bfloat16}[prec]
+    xt = torch.float64 if prec == "f64" else torch.float32
+    val = torch.ones(nnz, dtype=vt, device=dev)
+    if prec == "bf16":
+        val = val.view(torch.int16)
+    x = torch.ones(n, dtype=xt, device=dev)
+    y = torch.empty(m, dtype=xt, device=dev)
+    fn = {"f64": C.ssspmv_csr_f64, "f32": C.ssspmv_csr_f32, "bf16": C.ssspmv_csr_bf16f32}[prec]
+    us = []
+    for opts in (None, C.make_opts(variant=C.VARIANT_SPECULATIVE)):
+        us.append(_us(lambda: C.check(fn(m, n, nnz, rp, col, val, x, y, opts=opts), prec)))
+        assert torch.all(y == float(length))
+    assert us[0] <= 1.25 * us[1], us
