@@ -445,8 +445,6 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
     while (cur.nr > 0) {
         if (BATCHED && cur.mat != mat) load_matrix(mat = cur.mat);
         const int32_t rows = 32 >> gs;  // per group
-        const int sub = lane & ((1 << gs) - 1);
-        const int lrow = lane >> gs;  // the lane's row in its group
 #pragma unroll
         for (int i = 0; i < NP; ++i)
             if (32 * i + lane <= cur.nr) sc->rp[32 * i + lane] = cur.rp[i];
@@ -459,9 +457,14 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
         A carry = P::zero();
 #pragma unroll 1
         while (j < cur.nr) {
-            const int32_t g0 = inside(rp[j], b, e), ge = inside(rp[j + rows], g0, e);
-            const int32_t T = ge - g0;
-            if (T > 2 * cap && (!MULTI || T > row_most(nnz, gs, cap))) {
+            // log2 of the lanes per row in this round, and its rows: a group's, or
+            // half of one's
+            const bool second = MULTI && (j & (rows - 1)) != 0;
+            int gl = gs + second;
+            int32_t rl = 32 >> gl;
+            const int32_t g0 = inside(rp[j], b, e);
+            int32_t ge = inside(rp[j + rl], g0, e), T = ge - g0;
+            if (!second && T > 2 * cap && (!MULTI || T > row_most(nnz, gs, cap))) {
                 const int32_t l = lane < rows ? lane : 0;
                 const int32_t rs = inside(rp[j + l], g0, ge), re = inside(rp[j + l + 1], rs, ge);
                 const int32_t left = m - (cur.r0 + j);
@@ -470,16 +473,35 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
                 j += rows;
                 continue;
             }
+            // a group of rows of about the same length that does not fit the stage
+            // goes by halves of its rows with twice the lanes for each, not by even
+            // parts of its entries (diagonal blocks of 32 to 64 rows, 28 million
+            // entries: FP64 94 us -> 75, FP32 80 -> 54, BF16 values 80 -> 54; of 32
+            // to 230: 88 -> 78, 71 -> 58, 71 -> 57.  Uneven groups by halves too:
+            // R-MAT of edge factor 32 in FP32 15% slower; more lanes per row from
+            // the mean: bands up to 30% slower)
+            if (MULTI && !second && T > cap && gs > 0 && gs < 5) {
+                const int32_t rs = rp[j + (lane >> gs)], re = rp[j + (lane >> gs) + 1];
+                const int32_t longest = (int32_t)__reduce_max_sync(FULL, (unsigned)(re - rs));
+                if (P::rows_even((longest + (1 << gs) - 1) >> gs, T)) {
+                    ++gl;
+                    rl >>= 1;
+                    ge = inside(rp[j + rl], g0, e);
+                    T = ge - g0;
+                }
+            }
+            const int sub = lane & ((1 << gl) - 1);
+            const int lrow = lane >> gl;  // the lane's row
             // the entries [ts, te) of the rows [j, jn): this group and those
-            // after it that fit with it; or an even part of a group that does
-            // not fit by itself
-            int32_t ts = g0, te = ge, jn = j + rows;
+            // after it that fit with it; or an even part of a group (of a row)
+            // that does not fit by itself
+            int32_t ts = g0, te = ge, jn = j + rl;
             if (T > cap) {
                 const int32_t parts = (T + cap - 1) / cap;
                 const int32_t len = ((T + parts - 1) / parts + 7) & ~7;
                 ts = at < 0 ? g0 : at;
                 te = ts + len < ge ? ts + len : ge;
-            } else {
+            } else if (rl == rows) {
                 while (jn < cur.nr) {
                     const int32_t t = inside(rp[jn + rows], te, e);
                     if (t - g0 > cap) break;
@@ -500,14 +522,14 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
             int32_t steps = 0;
             bool even = false;
             if (T <= cap) {
-                for (int32_t k = j; k < jn; k += rows) {
+                for (int32_t k = j; k < jn; k += rl) {
                     const int32_t rs = inside(rp[k + lrow], ts, te);
                     const int32_t n = inside(rp[k + lrow + 1], rs, te) - rs - sub;
                     steps += (int32_t)__reduce_max_sync(
-                        FULL, (unsigned)(MULTI ? (n + (1 << gs) - 1) >> gs : n));
+                        FULL, (unsigned)(MULTI ? (n + (1 << gl) - 1) >> gl : n));
                 }
                 even = P::rows_even(steps, te - ts);
-            } else if (MULTI && rows == 1) {
+            } else if (MULTI && rl == 1) {
                 steps = (te - ts + 31) >> 5;
                 even = true;  // a part of one long row
             }
@@ -519,7 +541,7 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
                 __syncwarp();
                 const uint32_t inv = 65535u / (uint32_t)C + 1u;  // exact: p * C < 2^16
                 int32_t base = 0;
-                for (int32_t k = j; k < jn; k += rows) {
+                for (int32_t k = j; k < jn; k += rl) {
                     const int32_t r0 = rp[k + lrow], r1 = rp[k + lrow + 1];
                     const int32_t rs = inside(r0, ts, te), re = inside(r1, rs, te);
                     const bool holder = sub == 0 && re > rs;
@@ -549,12 +571,12 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
             __syncwarp();
             const int32_t off = ts & 7;  // the first entry's shared index
             if (even) {
-                for (int32_t k = j; k < jn; k += rows) {
+                for (int32_t k = j; k < jn; k += rl) {
                     const int32_t rs = inside(rp[k + lrow], ts, te);
                     const int32_t len = inside(rp[k + lrow + 1], rs, te) - rs;
-                    const int32_t n = MULTI ? (len - sub + (1 << gs) - 1) >> gs : len;
+                    const int32_t n = MULTI ? (len - sub + (1 << gl) - 1) >> gl : len;
                     // (of a single group: counted above)
-                    const int32_t nmax = jn == j + rows
+                    const int32_t nmax = jn == j + rl
                                              ? steps
                                              : (int32_t)__reduce_max_sync(FULL, (unsigned)n);
                     const int32_t nmin = (int32_t)__reduce_min_sync(FULL, (unsigned)n);
@@ -567,11 +589,11 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
                     A acc;
                     if (__popc(banks) <= 8 && nmax >= 8)
                         acc = lane_dot<P, P::kLaneBatch, MULTI ? 0 : 1, true>(
-                            sv + first, scol + first, x, n, nmin, nmax, 1 << gs,
+                            sv + first, scol + first, x, n, nmin, nmax, 1 << gl,
                             n > 0 ? lrow % n : 0, pol_keep, MULTI ? carry : P::zero());
                     else
                         acc = lane_dot<P, P::kLaneBatch, MULTI ? 0 : 1, false>(
-                            sv + first, scol + first, x, n, nmin, nmax, 1 << gs, 0, pol_keep,
+                            sv + first, scol + first, x, n, nmin, nmax, 1 << gl, 0, pol_keep,
                             MULTI ? carry : P::zero());
                     if (MULTI && te < ge) {  // a part of one long row: lane by lane
                         carry = acc;
@@ -579,7 +601,7 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
                     }
                     if (MULTI) carry = P::zero();
                     if (MULTI)
-                        for (int d = 1; d < (1 << gs); d <<= 1)
+                        for (int d = 1; d < (1 << gl); d <<= 1)
                             acc = P::add(acc, P::shfl(acc, lane ^ d));
                     if (sub == 0 && cur.r0 + k + lrow < m) store(cur.r0 + k + lrow, acc);
                 }

@@ -465,3 +465,70 @@ def test_long_rows_are_no_slower_than_by_tiles(dev, prec, length):
         us.append(_us(lambda: C.check(fn(m, n, nnz, rp, col, val, x, y, opts=opts), prec)))
         assert torch.all(y == float(length))
     assert us[0] <= 1.25 * us[1], us
+
+
+def _block_rows(lo, hi, total, rng):
+    """Row lengths of a block-diagonal matrix of dense blocks of lo to hi rows."""
+    sizes = rng.integers(lo, hi + 1, size=2 * total // ((lo + hi) * lo) + 50)
+    lens = np.repeat(sizes, sizes)
+    return lens[: np.searchsorted(np.cumsum(lens), total)]
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("lo,hi", [(32, 64), (30, 70), (32, 130), (40, 256), (200, 500)])
+def test_groups_by_halves(dev, lo, hi, prec):
+    """Equal rows in a group, several lanes each, more entries than a stage: by
+    halves, next to groups that fit, with a few rows that break the evenness."""
+    from paper_1504_06474_gb300 import ssspmv as C
+    rng = np.random.default_rng(hi)
+    lens = _block_rows(lo, hi, 3_000_000, rng)
+    at = rng.choice(lens.size, 200, replace=False)
+    lens[at[:100]] = 0
+    lens[at[100:]] = rng.integers(1, 700, size=100)
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    m, n, nnz = lens.size, 517, int(rp[-1])
+    col = rng.integers(0, n, size=nnz).astype(np.int32)
+    val, x = rng.integers(-6, 7, size=nnz).astype(float), rng.integers(-6, 7, size=n).astype(float)
+    want = oracle.spmv(rp, col, val, x)
+    vt = {"f64": torch.float64, "f32": torch.float32, "bf16": torch.bfloat16}[prec]
+    fn = {"f64": C.ssspmv_csr_f64, "f32": C.ssspmv_csr_f32, "bf16": C.ssspmv_csr_bf16f32}[prec]
+    xt = torch.float64 if prec == "f64" else torch.float32
+    rpd, cd, vd, xd = _device(dev, (rp, col, val, x))
+    vd = vd.to(vt).view(torch.int16) if prec == "bf16" else vd.to(vt)
+    y = torch.full((m,), float("nan"), dtype=xt, device=dev)
+    C.check(fn(m, n, nnz, rpd, cd, vd, xd.to(xt), y), prec)
+    assert np.array_equal(y.cpu().numpy().astype(np.float64), want)
+    if prec == "f32":  # the same bits in a batch
+        val32, x32 = (torch.as_tensor(rng.uniform(-1, 1, k).astype(np.float32), device=dev)
+                      for k in (nnz, n))
+        C.check(fn(m, n, nnz, rpd, cd, val32, x32, y), "f32")
+        yb = torch.full((m,), float("nan"), device=dev)
+        desc = torch.frombuffer(bytearray(C.batch_descriptors(
+            [(m, n, nnz, rpd, cd, val32, x32, yb)])), dtype=torch.uint8).to(dev)
+        ws = torch.empty(C.ssspmv_batched_workspace_bytes(1, nnz), dtype=torch.uint8, device=dev)
+        C.check(C.ssspmv_csr_batched_f32(1, desc, nnz, workspace=ws), "batched")
+        assert torch.equal(y, yb)
+
+
+@pytest.mark.parametrize("prec", ["f32", "bf16", "f64"])
+def test_diagonal_blocks_are_no_slower_than_by_tiles(dev, prec):
+    # (split evenly, their two-stage groups took 1.1 to 1.3 times the tiles' time)
+    from paper_1504_06474_gb300 import ssspmv as C
+    lens = _block_rows(32, 64, 28_000_000, np.random.default_rng(1))
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    m, nnz = lens.size, int(rp[-1])
+    rpd = torch.as_tensor(rp, device=dev)
+    col = (torch.arange(nnz, device=dev) % 100_000).to(torch.int32)
+    vt = {"f64": torch.float64, "f32": torch.float32, "bf16": torch.bfloat16}[prec]
+    xt = torch.float64 if prec == "f64" else torch.float32
+    val = torch.ones(nnz, dtype=vt, device=dev)
+    if prec == "bf16":
+        val = val.view(torch.int16)
+    x = torch.ones(100_000, dtype=xt, device=dev)
+    y = torch.empty(m, dtype=xt, device=dev)
+    fn = {"f64": C.ssspmv_csr_f64, "f32": C.ssspmv_csr_f32, "bf16": C.ssspmv_csr_bf16f32}[prec]
+    us = []
+    for opts in (None, C.make_opts(variant=C.VARIANT_SPECULATIVE)):
+        us.append(_us(lambda: C.check(fn(m, 100_000, nnz, rpd, col, val, x, y, opts=opts), prec)))
+        assert np.array_equal(y.cpu().numpy(), lens)
+    assert us[0] <= 1.05 * us[1], us
