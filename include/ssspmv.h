@@ -34,6 +34,11 @@
  *     asynchronous copies); x and y need only natural alignment.
  *   - Column indices must lie in [0, n); an out-of-range column is undefined
  *     behaviour (call ssspmv_validate_csr first for untrusted input).
+ *   - row_ptr must start at 0, never decrease and end at nnz.  The kernels stay
+ *     inside the arrays whatever it holds, but y is then not the product, and
+ *     not every such row_ptr is reported: the segmented sum over tiles flags
+ *     rows and counts that do not match, products by blocks of rows clamp each
+ *     row to the arrays and flag only more long rows than nnz entries can hold.
  *   - Return value: SSSPMV_OK (0) or a negative code; nothing is launched
  *     when a host-side check fails.  No C++ exception crosses the ABI.
  *   - The same input gives bit-identical y on every run (no floating-point
@@ -64,7 +69,8 @@ extern "C" {
 /* Device error bits written by the kernels into the workspace (read with
  * ssspmv_device_status). */
 #define SSSPMV_DEV_TIMEOUT   1u  /* a bounded wait on a bulk copy gave up */
-#define SSSPMV_DEV_RANGE     2u  /* a computed row index fell outside [0, m) */
+#define SSSPMV_DEV_RANGE     2u  /* a computed row index fell outside [0, m), or row_ptr has
+                                    more long rows than nnz entries can hold */
 #define SSSPMV_DEV_CALIB     4u  /* calibration found a segment count that does not match row_ptr */
 #define SSSPMV_DEV_BATCH     8u  /* a batch descriptor was invalid (that matrix was skipped) or
                                     the batch exceeded the capacity its workspace was sized for
@@ -155,7 +161,10 @@ size_t ssspmv_workspace_bytes(int32_t m, int32_t nnz, int32_t val_bytes, const s
  * library owns, cached per (device, stream) and grown stream-ordered with
  * cudaMallocAsync on `stream` when a call needs more (see
  * ssspmv_cached_workspace).  Kernels: by blocks of rows, or (a), (b), (c)
- * above (see SSSPMV_VARIANT_DEFAULT). */
+ * above (see SSSPMV_VARIANT_DEFAULT).  By blocks of rows a caller's buffer costs
+ * a 64-byte cudaMemsetAsync before the kernels, because it may hold anything;
+ * the library's own buffer (until its address is asked for) and a plan's are
+ * known to be clean.  The same holds for the other products below. */
 int ssspmv_csr_f64(int32_t m, int32_t n, int32_t nnz,
                    const int32_t *row_ptr, const int32_t *col_idx, const double *val,
                    const double *x, double *y,
@@ -273,7 +282,7 @@ int ssspmv_csr_batched_f32(int32_t count, const ssspmv_csr_desc *mats, int64_t t
 /* Learned variant selector (not in the paper; it only chooses among the
  * kernels above and never changes their arithmetic).
  *   ssspmv_features  16 statistics of row_ptr alone, each of order one, into
- *     device float[16] (one pass over the rows twice, then one thread):
+ *     device float[16] (one pass over the rows, finished by the last block):
  *     log2 m, log2 nnz, log2 mean row length, coefficient of variation of the
  *     lengths, log2 max length, fractions of empty rows, of rows <= 4, of
  *     rows >= 2x the mean, of entries in rows > 1024, median / 90th / 99th
@@ -324,8 +333,8 @@ int ssspmv_mlp_select(const float *params, const float *X, int32_t B, int32_t F,
  * bytes of synchronizer record per bunch of 4 -- i.e. nnz up to 223,671,840
  * at W = 15); options the other calls reject are rejected with the same
  * code.  All calls on a device share the array and it keeps the last call's
- * contents: each call clears its 16-byte header (error word, bunch ticket,
- * dirty-tile count, schedule flag) with cudaMemsetAsync on `stream`, and the
+ * contents: each call clears its 64-byte header (error words, tickets, list
+ * lengths, schedule flag) with cudaMemsetAsync on `stream`, and the
  * kernels write every other entry before reading it.  Calls that overlap on the GPU race
  * on the array -- order them on one stream.  The first call on a device
  * looks up the array's address (cudaGetSymbolAddress) with that device
