@@ -63,7 +63,7 @@ def peaks():
 # the sources that define the product's kernels and their launches (device code,
 # tile and row-block shapes, workspace carve-up); host-only files do not change
 # their traffic
-KERNEL_B_SOURCES = ("layout.h", "launch.cuh", "ptx.cuh", "rowblock.cuh", "rowshape.h",
+PRODUCT_SOURCES = ("layout.h", "launch.cuh", "ptx.cuh", "rowblock.cuh", "rowshape.h",
                     "segsum.cuh", "spmv_f64.cu")
 
 
@@ -97,11 +97,19 @@ def product_ms(path: dict, stages: dict) -> float:
     return sum(stages[n] for n in path["stages"] if n in ("rowblock", "rowtail", "segsum"))
 
 
+def tile_fields(path: dict, shape: dict, keys=("W", "L", "S", "bunches")) -> dict:
+    """The tile shape of a product, null where it goes by row blocks (which cut
+    out no tiles: ssspmv_plan_shape gives what the tiles would take)."""
+    names = {"bunches": "nbunches"}
+    return {k: None if path["kernel"] == "rowblock_kernel" else shape[names.get(k, k)]
+            for k in keys}
+
+
 def source_digest() -> str:
     import hashlib
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1504_06474_gb300", "csrc")
-    for name in KERNEL_B_SOURCES:
+    for name in PRODUCT_SOURCES:
         with open(os.path.join(csrc, name), "rb") as f:
             h.update(name.encode() + b"\0" + f.read())
     return h.hexdigest()[:16]
@@ -446,10 +454,10 @@ def run_ours(args):
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
             "data": "synthetic",
             "config": {"workload": args.workload, "m": A.m, "n": A.n, "nnz": A.nnz,
-                       "W": shape["W"], "L": shape["L"], "S": shape["S"],
+                       **tile_fields(path, shape),
                        "variant": ["default", "speculative", "exact", "rows"][args.variant],
                        "block_warps": args.block_warps, "selector": selected,
-                       "bunches": shape["nbunches"], "bytes_per_step": nbytes,
+                       "bytes_per_step": nbytes,
                        "ms_per_step_median": round(statistics.median(per_step), 5),
                        "paper_bytes_per_step": paper_bytes(A.m, A.nnz),
                        "hbm_frac": round(value / world / hbm, 4),
@@ -689,7 +697,8 @@ def measure_single(A, x, dev, precision, opts_kw, K, workload, cpu_seconds=0.0, 
         "dtype": {"f64": "f64", "f32": "f32", "bf16": "bf16-val/f32"}[precision],
         "data": "synthetic",
         "config": {"workload": workload, "precision": precision, "m": A.m, "n": A.n,
-                   "nnz": A.nnz, "W": shape["W"], "S": shape["S"], "bytes_per_step": nbytes,
+                   "nnz": A.nnz, **tile_fields(path, shape, ("W", "S")),
+                   "bytes_per_step": nbytes,
                    "hbm_frac": round(value / hbm, 4), "us_per_call": round(whole * 1e3, 2),
                    "ms_per_step_median": round(med, 5), "stage_ms": st,
                    "l2": ("not flushed (hot: inputs stay in L2 between steps)" if hot else
@@ -778,7 +787,7 @@ def _summary(line, keep_error=True):
     c = line["config"]
     out = {"value": line["value"], "unit": line["unit"], "dtype": line["dtype"],
            "ms_per_step": line["ms_per_step"], "hbm_frac": c.get("hbm_frac"),
-           "kernel_b_frac": line["roofline"]["frac"], "stage_ms": c.get("stage_ms"),
+           "kernels_frac": line["roofline"]["frac"], "stage_ms": c.get("stage_ms"),
            "steps": line["steps"], "clocks": line["clocks"], "l2": c.get("l2")}
     for k in ("us_per_call", "speedup_vs_plain_f64", "plain_f64_ms", "W", "S", "m", "nnz"):
         if k in c:
@@ -831,7 +840,7 @@ def extra_configs(args, dev):
     b = measure_batch(ns, dev)
     bs = {"value": b["value"], "unit": b["unit"], "dtype": b["dtype"],
           "ms_per_step": b["ms_per_step"], "hbm_frac": b["config"]["hbm_frac"],
-          "kernel_b_frac": b["roofline"]["frac"], "steps": b["steps"], "clocks": b["clocks"]}
+          "kernels_frac": b["roofline"]["frac"], "steps": b["steps"], "clocks": b["clocks"]}
     for k in ("matrices", "families", "rows", "nnz", "W", "variant", "autotuned", "launch",
               "stage_ms", "speedup_vs_separate_f32_calls", "speedup_vs_plain_f64",
               "separate_f32_calls_ms", "separate_plain_f64_calls_ms", "l2"):
@@ -1022,7 +1031,7 @@ def measure_batch(args, dev):
         "config": {"workload": args.workload, "matrices": count, "families": fams,
                    "rows": sum(A.m for A, _ in mats), "nnz": total_nnz,
                    "bytes_per_step": nbytes, "hbm_frac": round(value / hbm, 4),
-                   "W": C.ssspmv_plan_shape(1, 1, 4, opts)["W"],
+                   **tile_fields(path, C.ssspmv_plan_shape(1, 1, 4, opts), ("W",)),
                    "variant": ["default", "speculative", "exact", "rows"][args.variant],
                    "autotuned": tuned,
                    "launch": "one CUDA graph replay: set-up, then " + (

@@ -84,3 +84,14 @@ def test_traffic_record_follows_the_sources(tmp_path, monkeypatch):
     monkeypatch.setattr(bench, "source_digest", lambda: "0" * 16)   # sources changed since
     assert bench.ncu_traffic("segsum_kernel", "w") is None
 
+
+
+def test_tile_shape_is_null_by_row_blocks():
+    import bench
+    shape = {"W": 15, "L": 480, "S": 4, "ntiles": 12, "nbunches": 3}
+    rows = bench.product_path({"W": 0, "S": 0, "variant": 0, "block_warps": 0})
+    assert bench.tile_fields(rows, shape) == {"W": None, "L": None, "S": None, "bunches": None}
+    for kw in ({"W": 15}, {"variant": 1}, {"S": 2}):
+        got = bench.tile_fields(bench.product_path(kw), shape)
+        assert got == {"W": 15, "L": 480, "S": 4, "bunches": 3}
+    assert bench.tile_fields(bench.product_path({"variant": 3}), shape, ("W",)) == {"W": 15}
