@@ -289,7 +289,7 @@ def run_ours(args):
     if args.select:
         # the shipped network's class for this matrix, from its device features
         from paper_1504_06474_gb300 import selector as SEL
-        params = SEL.load_default()
+        params = SEL.load_current()
         if params is None:
             raise RuntimeError("no selector weights shipped with the package")
         f = SEL.device_features(Ad.row_ptr, A.m, A.n, A.nnz).cpu().numpy()[None, :]
@@ -762,7 +762,7 @@ def _select_compare(single, dev, K, flush_l2, gpu):
     import torch
     from paper_1504_06474_gb300 import selector as SEL
     from paper_1504_06474_gb300 import ssspmv as C
-    params = SEL.load_default()
+    params = SEL.load_current()
     if params is None:
         return {"unavailable": "no selector weights shipped with the package"}
     A = single.A

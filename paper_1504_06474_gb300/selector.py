@@ -1,8 +1,9 @@
 """Learned variant and tile-shape selector (not in the paper).
 
-The library has several ways to compute the same y = A x: the speculative
-segmented sum at four tile lengths, the exact-store variant, two warp counts,
-and the row-parallel kernels.  Which is fastest depends on the row structure.
+The library has several ways to compute the same y = A x: blocks of rows (its
+default), the speculative segmented sum at four tile lengths, the exact-store
+variant, two warp counts, and the row-parallel kernels.  Which is fastest depends
+on the row structure.
 This module
 
 * measures it: ``autotune`` times every class on a matrix on the GPU
@@ -13,10 +14,16 @@ This module
   class's time, trained on the GPU by the library's own FP32 forward,
   backward and Adam kernels (``ssspmv_mlp_*``);
 * chooses: the class of least predicted time (``ssspmv_mlp_select``); with no
-  model, or non-finite features, the plain speculative kernel (class 0, the
-  library's defaults) is the fallback.
+  model, with one that ranks other classes than ``CLASSES``, or with non-finite
+  features, class 0 (the library's defaults) is the fallback.
 
 The choice never changes the arithmetic of a class, only which class runs.
+
+Two sets of weights come with the package.  ``load_current()`` gives those that
+rank ``CLASSES``, trained on the kernels as they are: choose with these.
+``load_default()`` gives the first ones, for which class 0 was the tiles at
+W = 15; a stencil that they send to the tiles takes 1.13 times the default's time
+by now, so ``select`` and ``choose_opts`` take class 0 for them.
 
     python -m paper_1504_06474_gb300.selector --train 2000 --test 200 --out DIR
 
@@ -294,10 +301,28 @@ def train(X: np.ndarray, T: np.ndarray, dev, steps: int = 4000, lr: float = 3e-3
     return p.cpu().numpy()
 
 
+class Weights(np.ndarray):
+    """Parameters from a file, with the names of the classes they rank."""
+    classes = None
+
+    def __array_finalize__(self, obj):
+        self.classes = getattr(obj, "classes", None)
+
+
+def ranks_classes(params) -> bool:
+    """Whether these parameters rank CLASSES, as far as they say: those from a
+    file carry its class names, an array of a user's own does not."""
+    names = getattr(params, "classes", None)
+    return names is None or names == [c[0] for c in CLASSES]
+
+
 def select(params: np.ndarray, X: np.ndarray, dev) -> np.ndarray:
-    """Class per row of X; class 0 (the default) where a feature is not finite."""
-    import torch
+    """Class per row of X; class 0 (the default) where a feature is not finite,
+    and for parameters that rank other classes."""
     B = X.shape[0]
+    if not ranks_classes(params):
+        return np.zeros(B, np.int32)
+    import torch
     p = torch.as_tensor(np.ascontiguousarray(params, np.float32), device=dev)
     Xd = torch.as_tensor(np.nan_to_num(np.ascontiguousarray(X, np.float32)), device=dev)
     scratch = torch.empty(C.ssspmv_mlp_scratch_floats(B, F, H1, H2, K), dtype=torch.float32,
@@ -338,25 +363,40 @@ def load(path: str) -> np.ndarray:
         d = json.load(f)
     if d["dims"] != [F, H1, H2, K]:
         raise ValueError("selector weights for dims %s, expected %s" % (d["dims"], [F, H1, H2, K]))
-    return np.asarray(d["params"], np.float32)
+    p = np.asarray(d["params"], np.float32).view(Weights)
+    p.classes = d.get("classes")
+    return p
 
 
-DEFAULT_WEIGHTS = os.path.join(os.path.dirname(os.path.abspath(__file__)), "selector_weights.json")
+_HERE = os.path.dirname(os.path.abspath(__file__))
+DEFAULT_WEIGHTS = os.path.join(_HERE, "selector_weights.json")
+CURRENT_WEIGHTS = os.path.join(_HERE, "selector_weights_rows.json")
 
 
 def load_default():
-    """The weights trained by this module's command line on 2,000 generated
-    matrices (shipped with the package), or None if absent."""
+    """The first weights shipped with the package, trained when class 0 was the
+    tiles at W = 15 (see the module's notes), or None if absent."""
     try:
         return load(DEFAULT_WEIGHTS)
     except (OSError, ValueError, KeyError):
         return None
 
 
+def load_current():
+    """The weights that rank CLASSES, trained by this module's command line on
+    2,000 generated matrices (shipped with the package), or None if absent or
+    trained for other classes."""
+    try:
+        p = load(CURRENT_WEIGHTS)
+    except (OSError, ValueError, KeyError):
+        return None
+    return p if ranks_classes(p) else None
+
+
 def choose_opts(rp, m: int, n: int, nnz: int, params=None, timer=None):
-    """opts for ssspmv_csr_f64 on this matrix: the selector's class, or the
-    defaults when there is no model."""
-    if params is None:
+    """opts for ssspmv_csr_f64 on this matrix: the selector's class (params:
+    load_current()), or the defaults when there is no model for CLASSES."""
+    if params is None or not ranks_classes(params):
         return class_opts(0, timer)
     f = device_features(rp, m, n, nnz).cpu().numpy()[None, :]
     k = int(select(params, f, rp.device)[0])
