@@ -162,7 +162,7 @@ size_t ssspmv_workspace_bytes(int32_t m, int32_t nnz, int32_t val_bytes, const s
  * cudaMallocAsync on `stream` when a call needs more (see
  * ssspmv_cached_workspace).  Kernels: by blocks of rows, or (a), (b), (c)
  * above (see SSSPMV_VARIANT_DEFAULT).  By blocks of rows a caller's buffer costs
- * a 64-byte cudaMemsetAsync before the kernels, because it may hold anything;
+ * a launch that clears its header before the kernels, because it may hold anything;
  * the library's own buffer (until its address is asked for) and a plan's are
  * known to be clean.  The same holds for the other products below. */
 int ssspmv_csr_f64(int32_t m, int32_t n, int32_t nnz,

@@ -254,6 +254,18 @@ static int cached_workspace(size_t need, void *stream, void **ptr, size_t *bytes
     return SSSPMV_OK;
 }
 
+// The header words of a caller's workspace, which may hold anything, before the
+// row blocks.  A kernel of their chain of dependent launches: a memset between
+// them makes each wait for the one before to end (120,000 rows of 0..32 entries
+// 20.6 us a call, so 17.7; 4,096 rows under a CUDA graph 9.9 and 5.9; a call by
+// itself the same within 0.5).
+__global__ void clear_header_kernel(uint32_t *head)
+{
+    grid_dep_wait();
+    grid_dep_trigger();
+    head[threadIdx.x] = 0u;
+}
+
 // header: the state of the workspace's header words, kHeaderUnknown for a
 // caller's buffer
 enum { kHeaderUnknown = 0, kHeaderClear = 1 };
@@ -334,7 +346,9 @@ static int run_call(int32_t val_bytes, int32_t m, int32_t n, int32_t nnz,
     if (!tiles_only && takes_rows(val_bytes, m, nnz, opts, l)) {
         c.rows = 1;
         if (header != kHeaderClear) {
-            cudaError_t e = cudaMemsetAsync(c.ws + l.off_err, 0, kHeaderBytes, c.stream);
+            const cudaError_t e =
+                launch_dependent(clear_header_kernel, 1, (unsigned)kHeaderBytes / 4, 0, c.stream,
+                                 reinterpret_cast<uint32_t *>(c.ws + l.off_err));
             if (e != cudaSuccess) return record_cuda_error(e);
         }
     }
