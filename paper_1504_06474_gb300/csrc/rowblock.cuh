@@ -294,6 +294,20 @@ __device__ __forceinline__ void stage_copy(unsigned char *st, int32_t col_off, u
     }
 }
 
+// Whether a stage of T entries in `groups` groups, whose longest lanes take n
+// steps in all, keeps a lane per row (or G lanes), or splits its entries evenly
+// (T / 32 steps and the joining of the cut rows).  Each group adds a step for the
+// reductions that both ways make per group.  Against a longer lane of up to 2.5
+// times the mean and 15 for FP32: rows of 0..40, 0..80 and 0..160 entries, 30
+// million in all, FP32 139, 137 and 125 us and 123, 120 and 119 so, BF16 values
+// 130, 127, 118 and 118, 114, 114; that rule for FP64: 136, 131, 128 and 156, 152,
+// 137.  Without the step per group FP64 rows of 0..8 entries take 67 us instead of
+// 64 (10 million); with two or more, of 0..20 143 instead of 137 (30 million).
+__device__ __forceinline__ bool rows_even(int n, int T, int groups)
+{
+    return n <= (T >> 5) + (T >> 6) + 7 + groups;
+}
+
 // row pointer p as an index into [b, e], whatever row_ptr holds
 __device__ __forceinline__ int32_t inside(int32_t p, int32_t b, int32_t e)
 {
@@ -483,7 +497,7 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
             if (MULTI && !second && T > cap && gs > 0 && gs < 5) {
                 const int32_t rs = rp[j + (lane >> gs)], re = rp[j + (lane >> gs) + 1];
                 const int32_t longest = (int32_t)__reduce_max_sync(FULL, (unsigned)(re - rs));
-                if (P::rows_even((longest + (1 << gs) - 1) >> gs, T)) {
+                if (rows_even((longest + (1 << gs) - 1) >> gs, T, 1)) {
                     ++gl;
                     rl >>= 1;
                     ge = inside(rp[j + rl], g0, e);
@@ -522,13 +536,14 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
             int32_t steps = 0;
             bool even = false;
             if (T <= cap) {
-                for (int32_t k = j; k < jn; k += rl) {
+                int groups = 0;
+                for (int32_t k = j; k < jn; k += rl, ++groups) {
                     const int32_t rs = inside(rp[k + lrow], ts, te);
                     const int32_t n = inside(rp[k + lrow + 1], rs, te) - rs - sub;
                     steps += (int32_t)__reduce_max_sync(
                         FULL, (unsigned)(MULTI ? (n + (1 << gl) - 1) >> gl : n));
                 }
-                even = P::rows_even(steps, te - ts);
+                even = rows_even(steps, te - ts, groups);
             } else if (MULTI && rl == 1) {
                 steps = (te - ts + 31) >> 5;
                 even = true;  // a part of one long row

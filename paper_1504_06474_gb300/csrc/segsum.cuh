@@ -44,9 +44,6 @@ struct F64 {
     // 119, and stencil 160^3 245 instead of 239)
     static constexpr int kRowWarps = 19;
     static constexpr int kLaneBatch = 4, kSplitBatch = 4;  // gathers in flight per lane
-    // row blocks: a group of T entries whose longest lane takes n steps keeps
-    // a lane per row (or G lanes) rather than an even split of its entries
-    __device__ static __forceinline__ bool rows_even(int n, int T) { return n <= (T >> 5) + (T >> 6) + 8; }
     using val_t = double;
     using x_t = double;
     using y_t = double;
@@ -111,10 +108,6 @@ struct CompF32Traits {
     static constexpr int kRowWarps = 24;  // 80 registers
     // (eight or more in flight: more code and no faster)
     static constexpr int kLaneBatch = 4, kSplitBatch = 4;
-    __device__ static __forceinline__ bool rows_even(int n, int T)  // see F64
-    {
-        return 16 * n <= (T >> 5) * 40 + 240;
-    }
     using val_t = V;
     using x_t = float;
     using y_t = float;
