@@ -24,10 +24,10 @@
 // Measured (us a call among others; before: the three kernels of segsum.cuh).
 // FP64: 27-point stencil 160^3 272 -> 239 (the FP64 pipe alone needs 207), R-MAT
 // scale 22 with a 10^6-entry row 402 -> 327, banded half-width 31 (300,001 rows,
-// plan) 64 -> 51, uniform rows of 0..40 entries (120,007 rows, axpby) 40 -> 22,
+// plan) 64 -> 51, uniform rows of 0..40 entries (120,007 rows, axpby) 46 -> 22,
 // rows of 1..8 entries and three of 500,000 92 -> 62, uniform 4096 rows 15 -> 7.
-// FP32: stencil 101x97x103 62 -> 46, R-MAT scale 20 106 -> 89, 96 mixed matrices
-// 520 -> 337; BF16 values: stencil 120x125x131 110 -> 71.
+// FP32: stencil 101x97x103 62 -> 46, R-MAT scale 20 107 -> 89, 96 mixed matrices
+// 516 -> 344; BF16 values: stencil 120x125x131 110 -> 72.
 #pragma once
 #include <cstdint>
 
@@ -642,6 +642,13 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
 // warps, following the L1 that was left).
 
 constexpr int kTailThreads = 256;
+// Below this many entries two blocks per SM with eight entries per lane at a time,
+// from there on three with four.  Few very long rows in many short ones want the
+// former at any size measured (8 million entries, 3 rows of 500,000: 58 us and 65;
+// 12 million: 75 and 82), as do all matrices up to 5 million (R-MAT scale 16 of
+// edge factor 16 19 us and 22, longrows of 4 million 38 and 44); power laws above
+// 5.5 million the latter (R-MAT of 8 to 12 million 65 to 100 us and 61 to 93, of
+// 66 million 330 and 309; FP32 289 and 266).
 constexpr int32_t kTailWide = 15000000;
 constexpr int kTailShort = 24;    // rows up to this long: one lane each
 
@@ -1043,7 +1050,6 @@ int run_rowblock(const Call &c)
     if (rc) return rc;
     if (c.ev && (e = cudaEventRecord(c.ev[2], c.stream)) != cudaSuccess)
         rc = record_cuda_error(e);
-    // small matrices: fewer, longer rounds of loads per row
     if (!rc) rc = c.nnz < kTailWide ? launch_rowtail<P, 8, 2>(c, a) : launch_rowtail<P, 4, 3>(c, a);
     if (rc) {
         // (r1) has run and (r2) will not (its first launch loads it, and may find

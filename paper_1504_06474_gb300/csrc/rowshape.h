@@ -63,6 +63,8 @@ SSSPMV_HD inline RowShape row_shape(int32_t m, int32_t nnz, int32_t val_bytes)
     if (cap < kMinCap) cap = kMinCap;
     if (cap > kStageMax) cap = kStageMax;
     s.cap = (int32_t)cap;
+    // the lists have to fit the tiles' sections, which shrink per entry from
+    // 15.7 million entries on (several tiles per bunch): twice as long pieces then
     s.piece = nnz <= 15000000 ? kMinPiece : kMinPiece + 1;
     return s;
 }

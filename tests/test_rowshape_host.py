@@ -29,6 +29,11 @@ void shape(int32_t m, int32_t nnz, int32_t val_bytes, int32_t *out)
     out[4] = u.nbig;
     out[5] = u.nunits;
 }
+int64_t lists(int32_t m, int32_t nnz, int32_t val_bytes)
+{
+    const RowShape s = row_shape(m, nnz, val_bytes);
+    return (int64_t)row_lists(nnz, s.cap, s.piece).bytes;
+}
 }
 """
 
@@ -103,3 +108,22 @@ def test_short_rows_are_few_units(lib):
                           (20_000_000, 20, 185_000), (2_000_000, 1, 20_500)):
         s = _shape(lib, m, m * mean, 8)
         assert s["us"] == 2 and s["nunits"] <= most, (m, mean, s)
+
+
+def test_the_lists_fit_every_workspace(lib):
+    # (the header takes the first 256 bytes; with less room a product would go by
+    # tiles, see takes_rows)
+    import random
+    from paper_1504_06474_gb300 import _build
+    from paper_1504_06474_gb300 import ssspmv as C
+    _build.build()
+    lib.lists.restype = ctypes.c_int64
+    rng = random.Random(2)
+    for i in range(30_000):
+        m = int(2 ** rng.uniform(0, 31)) - 1
+        nnz = int(2 ** rng.uniform(0, 31)) - 1
+        if i < 3000:  # around the step in the pieces' length
+            nnz = 15_000_000 + rng.randint(-2000, 800_000)
+        m, nnz = min(max(m, 1), MAX_DIM), min(max(nnz, 1), MAX_DIM)
+        vb = rng.choice((8, 4, 2))
+        assert lib.lists(m, nnz, vb) <= C.ssspmv_workspace_bytes(m, nnz, vb, None) - 256, (m, nnz, vb)
