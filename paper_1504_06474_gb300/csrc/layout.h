@@ -132,13 +132,13 @@ inline void batch_layout(int32_t count, int64_t total_nnz, int32_t W, int32_t S,
 }
 
 // adds the row blocks' sections: the batch's entries are at most
-// cap_tiles * L, groups of more than 2 * min_cap of them are listed, in pieces
+// cap_tiles * L, groups of more than min_cap of them may be listed, in pieces
 // of at least 2^min_piece
 inline void batch_rows_layout(int32_t count, int32_t min_cap, int32_t min_piece, BatchLayout &l)
 {
     const int64_t nnz = l.cap_tiles * l.L;
     l.rows = 1;
-    l.cap_ranges = nnz / (2 * min_cap) + (nnz >> min_piece) + count + 1;
+    l.cap_ranges = nnz / min_cap + (nnz >> min_piece) + count + 1;
     l.cap_pieces = ((2 * nnz) >> min_piece) + count + 1;
     size_t o = l.total;
     auto take = [&](size_t bytes) {

@@ -478,30 +478,44 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
             int32_t rl = 32 >> gl;
             const int32_t g0 = inside(rp[j], b, e);
             int32_t ge = inside(rp[j + rl], g0, e), T = ge - g0;
-            if (!second && T > 2 * cap && (!MULTI || T > row_most(nnz, gs, cap))) {
-                const int32_t l = lane < rows ? lane : 0;
-                const int32_t rs = inside(rp[j + l], g0, ge), re = inside(rp[j + l + 1], rs, ge);
-                const int32_t left = m - (cur.r0 + j);
-                list_group(a, cur.mat, piece, cur.r0 + j, left < rows ? left : rows,
-                           lane < rows ? re - rs : 0);
-                j += rows;
-                continue;
-            }
-            // a group of rows of about the same length that does not fit the stage
-            // goes by halves of its rows with twice the lanes for each, not by even
-            // parts of its entries (diagonal blocks of 32 to 64 rows, 28 million
-            // entries: FP64 94 us -> 75, FP32 80 -> 54, BF16 values 80 -> 54; of 32
-            // to 230: 88 -> 78, 71 -> 58, 71 -> 57.  Uneven groups by halves too:
-            // R-MAT of edge factor 32 in FP32 15% slower; more lanes per row from
-            // the mean: bands up to 30% slower)
-            if (MULTI && !second && T > cap && gs > 0 && gs < 5) {
-                const int32_t rs = rp[j + (lane >> gs)], re = rp[j + (lane >> gs) + 1];
-                const int32_t longest = (int32_t)__reduce_max_sync(FULL, (unsigned)(re - rs));
-                if (rows_even((longest + (1 << gs) - 1) >> gs, T, 1)) {
-                    ++gl;
-                    rl >>= 1;
-                    ge = inside(rp[j + rl], g0, e);
-                    T = ge - g0;
+            // Listed: a group of too many entries, or (FP64) one that does not fit the
+            // stage and whose longest row has half of its entries: the two stages of
+            // such a group hold up its unit, and at the end of the launch all.  1,000
+            // rows of 1,000 entries in 166,666 of 4.5 on average 31 us, and listed 22,
+            // in 1.7 million 72 and 61; the row lengths of a Pareto law over 2,000 to
+            // 16,000 rows 18 to 23 us and 15 to 19.  (100 such rows in 5 million: 136
+            // and 144.  In FP32, where single and batched products have to agree, the
+            // test alone made 27-point stencils 3% slower.)
+            if (T > cap && !second) {
+                bool list = T > 2 * cap && (!MULTI || T > row_most(nnz, gs, cap));
+                if (!list && (sizeof(V) == 8 || MULTI) && gs < 5) {
+                    const int32_t rs = rp[j + (lane >> gs)], re = rp[j + (lane >> gs) + 1];
+                    const int32_t longest = (int32_t)__reduce_max_sync(FULL, (unsigned)(re - rs));
+                    list = sizeof(V) == 8 && longest >= T - longest;
+                    // a group of rows of about the same length that does not fit the
+                    // stage goes by halves of its rows with twice the lanes for each,
+                    // not by even parts of its entries (diagonal blocks of 32 to 64
+                    // rows, 28 million entries: FP64 94 us -> 75, FP32 80 -> 54, BF16
+                    // values 80 -> 54; of 32 to 230: 88 -> 78, 71 -> 58, 71 -> 57.
+                    // Uneven groups by halves too: R-MAT of edge factor 32 in FP32 15%
+                    // slower; more lanes per row from the mean: bands up to 30% slower)
+                    if (MULTI && !list && gs > 0 &&
+                        rows_even((longest + (1 << gs) - 1) >> gs, T, 1)) {
+                        ++gl;
+                        rl >>= 1;
+                        ge = inside(rp[j + rl], g0, e);
+                        T = ge - g0;
+                    }
+                }
+                if (list) {
+                    const int32_t l = lane < rows ? lane : 0;
+                    const int32_t rs = inside(rp[j + l], g0, ge);
+                    const int32_t re = inside(rp[j + l + 1], rs, ge);
+                    const int32_t left = m - (cur.r0 + j);
+                    list_group(a, cur.mat, piece, cur.r0 + j, left < rows ? left : rows,
+                               lane < rows ? re - rs : 0);
+                    j += rows;
+                    continue;
                 }
             }
             const int sub = lane & ((1 << gl) - 1);

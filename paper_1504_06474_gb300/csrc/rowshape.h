@@ -86,9 +86,9 @@ SSSPMV_HD inline int32_t row_most(int32_t nnz, int32_t gs, int32_t cap)
     return share < 8 * cap ? share : 8 * cap;
 }
 
-// bounds of the lists (r1) writes: at most one range of rows per `piece`
-// entries or part of it of an oversized group, and rows longer than a piece
-// cut into pieces
+// bounds of the lists (r1) writes, from groups of more than cap entries: at most
+// one range of rows per `piece` entries or part of it of such a group, and rows
+// longer than a piece cut into pieces
 struct RowLists {
     int64_t ranges, pieces;
     size_t off_ranges, off_pieces, off_parts, off_arrived, bytes;  // from the lists' start
@@ -97,7 +97,7 @@ struct RowLists {
 SSSPMV_HD inline RowLists row_lists(int64_t nnz, int32_t cap, int32_t piece)
 {
     RowLists l;
-    l.ranges = nnz / (2 * cap) + (nnz >> piece) + 1;
+    l.ranges = nnz / cap + (nnz >> piece) + 1;
     l.pieces = ((2 * nnz) >> piece) + 1;
     size_t o = 0;
     l.off_ranges = o;

@@ -532,3 +532,37 @@ def test_diagonal_blocks_are_no_slower_than_by_tiles(dev, prec):
         us.append(_us(lambda: C.check(fn(m, 100_000, nnz, rpd, col, val, x, y, opts=opts), prec)))
         assert np.array_equal(y.cpu().numpy(), lens)
     assert us[0] <= 1.05 * us[1], us
+
+
+@pytest.mark.parametrize("m,long,every", [(64_000, 641, 64), (64_003, 639, 64), (200_000, 700, 128),
+                                          (20_007, 1200, 96), (500_000, 1024, 352),
+                                          (500_000, 1025, 352)])
+def test_groups_that_one_row_fills(dev, m, long, every):
+    """Groups just past the stage whose longest row has most of the entries, as
+    many as the lists are sized for, between groups of short rows and empty ones."""
+    from paper_1504_06474_gb300 import ssspmv as C
+    rng = np.random.default_rng(every)
+    lens = rng.integers(0, 2, size=m) * (np.arange(m) % every >= 32)
+    lens[7::every] = long
+    lens[9::every] = 1
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    n, nnz = 517, int(rp[-1])
+    col = rng.integers(0, n, size=nnz).astype(np.int32)
+    val, x = rng.integers(-6, 7, size=nnz).astype(float), rng.integers(-6, 7, size=n).astype(float)
+    want = oracle.spmv(rp, col, val, x)
+    rpd, cd, vd, xd = _device(dev, (rp, col, val, x))
+    ws = torch.full((C.ssspmv_workspace_bytes(m, nnz, 8, None) + 256,), 255, dtype=torch.uint8,
+                    device=dev)
+    size = C.ssspmv_workspace_bytes(m, nnz, 8, None)
+    for _ in range(2):
+        y = torch.full((m,), float("nan"), dtype=torch.float64, device=dev)
+        C.check(C.ssspmv_csr_f64(m, n, nnz, rpd, cd, vd, xd, y, workspace=ws, ws_bytes=size), "csr")
+        assert C.ssspmv_device_status(ws) == 0
+        assert np.array_equal(y.cpu().numpy(), want)
+        assert bool((ws[size:] == 255).all())  # nothing past the workspace
+    C.check(C.ssspmv_csr_f64_axpby(m, n, nnz, rpd, cd, vd, xd, y, 2.0, -3.0, workspace=ws,
+                                   ws_bytes=size), "axpby")
+    assert np.array_equal(y.cpu().numpy(), -want)
+    y32 = torch.full((m,), float("nan"), device=dev)
+    C.check(C.ssspmv_csr_f32(m, n, nnz, rpd, cd, vd.float(), xd.float(), y32), "f32")
+    assert np.array_equal(y32.cpu().numpy().astype(np.float64), want)
