@@ -120,6 +120,18 @@ __device__ __forceinline__ typename P::acc_t lane_dot(const typename P::val_t *v
 constexpr int kTurnUnits = 8192;  // fewer units are all taken by turns
 constexpr int kUnitRowsMax = 128;
 constexpr int kBatchRowWarps = 20;  // a batch's kernel needs 96 registers
+// A kernel of its own for large matrices of very short rows: a stage of up to four
+// groups whose rows have no more than kShortRow entries is worked off at once,
+// where the general loop gathers for one group after the other, each a round trip
+// of some 0.8 us for 32 rows.  20 million rows, FP64: of one entry 277 us and 181
+// (the tiles 213), of 0 or 1 260 and 178 (209), of two 299 and 210 (285), of 1 to 3
+// 314 and 228 (287); FP32 223 and 148 (197), 198 and 147 (200), 237 and 168 (241),
+// 250 and 188 (245); 2 million of one entry 27.1 and 23.3; random columns from two
+// entries on and R-MATs from 2 million rows on the same within 2%.  (Below: R-MATs
+// of 0.5 and 1 million rows 2 to 5% slower, rows of one entry 7% faster.  In the
+// general kernel the loop costs longer rows more than it gives these.)
+constexpr int kShortRow = 4;
+constexpr int32_t kShortRows = 1500000;  // rows from which on it is taken
 
 struct alignas(16) RowScratch {
     uint64_t bar;
@@ -335,7 +347,7 @@ __device__ __forceinline__ int32_t find_matrix(const RowMat *mats, int32_t count
     return lo;
 }
 
-template <class P, bool MULTI, bool BATCHED = false>
+template <class P, bool MULTI, bool BATCHED = false, bool SHORT = false>
 __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32, 1)
     rowblock_kernel(const RowArgs a, int32_t stage_bytes, int32_t col_off)
 {
@@ -599,7 +611,44 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
             phase ^= 1u;
             __syncwarp();
             const int32_t off = ts & 7;  // the first entry's shared index
-            if (even) {
+            bool done = false;
+            if constexpr (SHORT) {
+                // up to four groups at once, so that their gathers overlap
+                constexpr int GM = kUnitRowsMax / 32;
+                int first[GM], n[GM], longest = 0;
+#pragma unroll
+                for (int g = 0; g < GM; ++g) {
+                    const int32_t r = j + 32 * g < jn ? j + 32 * g + lane : j;
+                    const int32_t rs = inside(rp[r], ts, te);
+                    n[g] = j + 32 * g < jn ? inside(rp[r + 1], rs, te) - rs : 0;
+                    first[g] = rs - ts + off;
+                    longest = n[g] > longest ? n[g] : longest;
+                }
+                const int nmax = (int)__reduce_max_sync(FULL, (unsigned)longest);
+                if (even && nmax <= kShortRow) {
+                    A acc[GM];
+#pragma unroll
+                    for (int g = 0; g < GM; ++g) acc[g] = P::zero();
+                    for (int i = 0; i < nmax; ++i) {
+                        X xv[GM];
+#pragma unroll
+                        for (int g = 0; g < GM; ++g)
+                            if (i < n[g]) xv[g] = P::gather(x, scol[first[g] + i], pol_keep);
+#pragma unroll
+                        for (int g = 0; g < GM; ++g)
+                            if (i < n[g]) acc[g] = P::fma(sv[first[g] + i], xv[g], acc[g]);
+                    }
+#pragma unroll
+                    for (int g = 0; g < GM; ++g) {
+                        const int32_t r = j + 32 * g + lane;
+                        if (j + 32 * g < jn && cur.r0 + r < m) store(cur.r0 + r, acc[g]);
+                    }
+                    done = true;
+                }
+            }
+            if (done) {
+                // stored above
+            } else if (even) {
                 for (int32_t k = j; k < jn; k += rl) {
                     const int32_t rs = inside(rp[k + lrow], ts, te);
                     const int32_t len = inside(rp[k + lrow + 1], rs, te) - rs;
@@ -969,11 +1018,11 @@ cudaError_t allow_smem(K kernel, int (&done)[64])
     return e;
 }
 
-template <class P, bool MULTI, bool BATCHED = false>
+template <class P, bool MULTI, bool BATCHED = false, bool SHORT = false>
 int launch_rowblock(const Call &c, const RowArgs &a)
 {
     static int done[64] = {0};
-    cudaError_t e = allow_smem(rowblock_kernel<P, MULTI, BATCHED>, done);
+    cudaError_t e = allow_smem(rowblock_kernel<P, MULTI, BATCHED, SHORT>, done);
     if (e != cudaSuccess) return record_cuda_error(e);
     // A gather that misses L1 holds one of its lines until it is served, so L1
     // has to be large enough for the gathers in flight: with all of shared
@@ -990,7 +1039,7 @@ int launch_rowblock(const Call &c, const RowArgs &a)
     const unsigned grid = (unsigned)(a.nunits < sms ? a.nunits : sms);
     const int32_t need = (int32_t)((a.nunits + (int64_t)grid - 1) / grid);
     if (warps > need) warps = need;
-    e = launch_dependent(rowblock_kernel<P, MULTI, BATCHED>, grid, (unsigned)warps * 32,
+    e = launch_dependent(rowblock_kernel<P, MULTI, BATCHED, SHORT>, grid, (unsigned)warps * 32,
                          (size_t)warps * (s.bytes + sizeof(RowScratch)), c.stream, a, s.bytes,
                          s.col_off);
     return e == cudaSuccess ? SSSPMV_OK : record_cuda_error(e);
@@ -1060,7 +1109,11 @@ int run_rowblock(const Call &c)
     a.alpha = c.alpha;
     a.beta = c.beta;
     a.axpby = c.axpby;
-    int rc = a.shape.gs > 0 ? launch_rowblock<P, true>(c, a) : launch_rowblock<P, false>(c, a);
+    int rc = SSSPMV_OK;
+    if (a.shape.gs > 0) rc = launch_rowblock<P, true>(c, a);
+    else if (c.m >= kShortRows && (int64_t)c.nnz <= 3 * (int64_t)c.m)
+        rc = launch_rowblock<P, false, false, true>(c, a);
+    else rc = launch_rowblock<P, false>(c, a);
     if (rc) return rc;
     if (c.ev && (e = cudaEventRecord(c.ev[2], c.stream)) != cudaSuccess)
         rc = record_cuda_error(e);

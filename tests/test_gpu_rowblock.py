@@ -566,3 +566,72 @@ def test_groups_that_one_row_fills(dev, m, long, every):
     y32 = torch.full((m,), float("nan"), device=dev)
     C.check(C.ssspmv_csr_f32(m, n, nnz, rpd, cd, vd.float(), xd.float(), y32), "f32")
     assert np.array_equal(y32.cpu().numpy().astype(np.float64), want)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("m", [1_499_999, 1_500_000, 1_700_003])
+def test_very_short_rows(dev, m, prec):
+    """Both sides of the size from which matrices of very short rows have a
+    kernel of their own: rows past its limit, uneven stages, listed groups and
+    empty stretches among them, and in FP32 the bits of the batch."""
+    from paper_1504_06474_gb300 import ssspmv as C
+    rng = np.random.default_rng(m)
+    n = 60_000
+    lens = rng.integers(0, 4, size=m)
+    lens[100_000:300_000] = rng.integers(0, 9, size=200_000)
+    lens[rng.choice(m, 3000, replace=False)] = 40
+    lens[rng.choice(m, 50, replace=False)] = rng.integers(300, 5000, size=50)
+    lens[400_000:420_000] = 0
+    lens[-40:] = 4
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    nnz = int(rp[-1])
+    assert nnz <= 3 * m
+    col = rng.integers(0, n, size=nnz).astype(np.int32)
+    val, x = rng.integers(-6, 7, size=nnz).astype(float), rng.integers(-6, 7, size=n).astype(float)
+    want = oracle.spmv(rp, col, val, x)
+    vt = {"f64": torch.float64, "f32": torch.float32, "bf16": torch.bfloat16}[prec]
+    fn = {"f64": C.ssspmv_csr_f64, "f32": C.ssspmv_csr_f32, "bf16": C.ssspmv_csr_bf16f32}[prec]
+    xt = torch.float64 if prec == "f64" else torch.float32
+    rpd, cd, vd, xd = _device(dev, (rp, col, val, x))
+    vd = vd.to(vt).view(torch.int16) if prec == "bf16" else vd.to(vt)
+    y = torch.full((m,), float("nan"), dtype=xt, device=dev)
+    C.check(fn(m, n, nnz, rpd, cd, vd, xd.to(xt), y), prec)
+    assert np.array_equal(y.cpu().numpy().astype(np.float64), want)
+    if prec == "f32":
+        val32, x32 = (torch.as_tensor(rng.uniform(-1, 1, k).astype(np.float32), device=dev)
+                      for k in (nnz, n))
+        C.check(fn(m, n, nnz, rpd, cd, val32, x32, y), "f32")
+        yb = torch.full((m,), float("nan"), device=dev)
+        desc = torch.frombuffer(bytearray(C.batch_descriptors(
+            [(m, n, nnz, rpd, cd, val32, x32, yb)])), dtype=torch.uint8).to(dev)
+        ws = torch.empty(C.ssspmv_batched_workspace_bytes(1, nnz), dtype=torch.uint8, device=dev)
+        C.check(C.ssspmv_csr_batched_f32(1, desc, nnz, workspace=ws), "batched")
+        assert torch.equal(y, yb)
+    elif prec == "f64":
+        C.check(C.ssspmv_csr_f64_axpby(m, n, nnz, rpd, cd, vd, xd, y, 2.0, -3.0), "axpby")
+        assert np.array_equal(y.cpu().numpy(), -want)
+        x_nan = x.copy()  # one column's NaN reaches exactly the rows that use it
+        x_nan[123] = np.nan
+        C.check(fn(m, n, nnz, rpd, cd, vd, torch.as_tensor(x_nan, device=dev), y), "nan")
+        uses = np.zeros(m, bool)
+        uses[np.repeat(np.arange(m), lens)[col == 123]] = True
+        assert np.array_equal(np.isnan(y.cpu().numpy()), uses)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_rows_of_one_entry_are_no_slower_than_by_tiles(dev, prec):
+    # (one group after the other, 20 million rows took 1.1 to 1.6 times the tiles' time)
+    from paper_1504_06474_gb300 import ssspmv as C
+    m = 20_000_000
+    xt = torch.float64 if prec == "f64" else torch.float32
+    rp = torch.arange(m + 1, device=dev, dtype=torch.int32)
+    col = torch.arange(m - 1, -1, -1, device=dev, dtype=torch.int32)
+    val = torch.full((m,), 2.0, dtype=xt, device=dev)
+    x = torch.arange(m, device=dev).to(xt)
+    y = torch.empty(m, dtype=xt, device=dev)
+    fn = C.ssspmv_csr_f64 if prec == "f64" else C.ssspmv_csr_f32
+    us = []
+    for opts in (None, C.make_opts(variant=C.VARIANT_SPECULATIVE)):
+        us.append(_us(lambda: C.check(fn(m, m, m, rp, col, val, x, y, opts=opts), prec)))
+        assert torch.equal(y, 2.0 * x.flip(0))
+    assert us[0] <= 1.05 * us[1], us
