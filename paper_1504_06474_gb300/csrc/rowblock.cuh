@@ -7,8 +7,9 @@
 //                         ones) are one contiguous range of the arrays, copied
 //                         to shared memory by two bulk copies.
 //   (r2) rowtail_kernel   groups of more entries than two stages hold (rows of
-//                         thousands of entries and their neighbours), listed
-//                         by (r1): a warp per row, or per piece of a very long
+//                         thousands of entries and their neighbours; in FP64
+//                         also smaller ones that one row fills), listed by
+//                         (r1): a warp per row, or per piece of a very long
 //                         row, straight from global memory.
 //
 // Why rows and not tiles of equal length: on this GPU one warp-wide FP64
@@ -483,7 +484,7 @@ __global__ void __launch_bounds__((BATCHED ? kBatchRowWarps : P::kRowWarps) * 32
         A carry = P::zero();
 #pragma unroll 1
         while (j < cur.nr) {
-            // log2 of the lanes per row in this round, and its rows: a group's, or
+            // log2 of the lanes per row in this pass, and its rows: a group's, or
             // half of one's
             const bool second = MULTI && (j & (rows - 1)) != 0;
             int gl = gs + second;
